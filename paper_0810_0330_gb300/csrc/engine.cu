@@ -67,6 +67,14 @@ struct seed_ctx {
   CsrOp csr{};
   WilsonOp wil{};
   int32_t *nbr = nullptr;
+  // Wilson: the FP64 operator in fixed-point arithmetic (wilson_fixed.cuh).  flinks / fexp are
+  // filled from the caller's links by every call that applies the operator; F and T hold the
+  // blocks of A's input and of D's output, Fe their exponents (F's columns, then T's).
+  WilsonFix wfix{};
+  int4 *flinks = nullptr, *F = nullptr;
+  int32_t *fexp = nullptr, *Fe = nullptr;
+  bool links_ready = false;            // flinks hold the links of the current call
+  double *dotpart = nullptr;           // partial sums of p^H q by 16 sites (wilson_fixed.cu)
 
   // seed recurrence
   void *V = nullptr;
@@ -228,6 +236,7 @@ seed_status alloc_common(seed_ctx *ctx) {
   const size_t es = ctx->vsz;
   const int m = ctx->prm.m_max;
   ctx->ldv = (n + 31) / 32 * 32;   // 256-byte aligned columns for complex, 256 B for real
+  if (ctx->kind == 1) ctx->ldv = (n / 12 + 31) / 32 * 384;   // whole 32-site tiles
   TRY(dalloc(ctx, &ctx->V, (size_t)ctx->ldv * (m + 1) * es));
   TRY(dalloc(ctx, &ctx->u, n * es));
   TRY(dalloc(ctx, &ctx->f, n * es));
@@ -295,8 +304,12 @@ GridSync grid_sync_bufs(seed_ctx *ctx) {
 seed_status ensure_cols(seed_ctx *ctx, int cols) {
   if (cols <= ctx->cap_cols) return SEED_OK;
   cudaStreamSynchronize(ctx->cs);
-  cudaFree(ctx->R); cudaFree(ctx->P); cudaFree(ctx->Q); cudaFree(ctx->T);
+  cudaFree(ctx->R); cudaFree(ctx->P); cudaFree(ctx->Q); cudaFree(ctx->T); cudaFree(ctx->F); cudaFree(ctx->Fe);
+  cudaFree(ctx->dotpart);
   ctx->R = ctx->P = ctx->Q = ctx->T = nullptr;
+  ctx->F = nullptr;
+  ctx->Fe = nullptr;
+  ctx->dotpart = nullptr;
   cudaFree(ctx->R32); cudaFree(ctx->P32); cudaFree(ctx->Q32); cudaFree(ctx->T32); cudaFree(ctx->E32);
   ctx->R32 = ctx->P32 = ctx->Q32 = ctx->T32 = ctx->E32 = nullptr;
   ctx->cap_cols = 0;
@@ -320,15 +333,58 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
   return SEED_OK;
 }
 
+// What the fixed-point operator needs, for a call that uses it (never inside a graph capture): its
+// work space for the context's columns, and the copy of the caller's links, once per call (the
+// caller may have changed them since the last one).
+seed_status ensure_fixed(seed_ctx *ctx) {
+  if (ctx->kind != 1 || ctx->links_ready) return SEED_OK;
+  const size_t cols = ctx->cap_cols;
+  if (!ctx->F) TRY(dalloc(ctx, &ctx->F, (size_t)ctx->ldv * cols * sizeof(int4)));
+  if (!ctx->Fe) TRY(dalloc(ctx, &ctx->Fe, sizeof(int32_t) * 2 * (size_t)(ctx->ldv / 12) * cols));
+  if (!ctx->dotpart) TRY(dalloc(ctx, &ctx->dotpart, sizeof(double) * (size_t)(ctx->ldv / 192) * cols));
+  launch_fix_links(ctx->wfix, ctx->cs);
+  ctx->links_ready = true;
+  ctx->stats.kernel_launches += 1;
+  return SEED_OK;
+}
+
+// T's columns hold blocks (16 bytes per component, like its doubles); Te: their exponents
+int4 *fix_T(seed_ctx *ctx) { return reinterpret_cast<int4 *>(ctx->T); }
+int32_t *fix_Te(seed_ctx *ctx) { return ctx->Fe + ctx->ldv / 12 * ctx->cap_cols; }
+
+// Y = A X on ncols columns in FP64 arithmetic throughout.  The Lanczos steps of the seed system take
+// this form: they amplify a last-bit change of A v_i until the late basis vectors, and through
+// the Galerkin projection the error (not the size) of the seeded solutions, differ by a per cent.
+int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols) {
+  if (ctx->kind == 0) {
+    launch_csr_spmv(ctx->csr, (const double *)X, ldx, (double *)Y, ldy, ncols, nullptr, ctx->cs);
+    return 1;
+  }
+  launch_wilson_dslash(ctx->wil, +1, (const double2 *)X, ldx, (double2 *)ctx->T, ctx->ldv, ncols, nullptr, ctx->cs);
+  launch_wilson_dslash(ctx->wil, -1, (const double2 *)ctx->T, ctx->ldv, (double2 *)Y, ldy, ncols, nullptr, ctx->cs);
+  return 2;
+}
+
 // Y = A X on ncols columns (mask: skip columns whose flag is 0).  Returns the kernel count.
+// Wilson: in fixed-point arithmetic from one tile per SM on; below that the FP64 kernel's two
+// launches (7 us each, one tile's FP64 instructions on its SM) are the shorter chain.
+bool fix_pays(const seed_ctx *ctx, int ncols) { return ctx->kind == 1 && ctx->ldv / 384 * ncols > ctx->sm_count; }
 int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, const int32_t *mask) {
   if (ctx->kind == 0) {
     launch_csr_spmv(ctx->csr, (const double *)X, ldx, (double *)Y, ldy, ncols, mask, ctx->cs);
     return 1;
   }
-  launch_wilson_dslash(ctx->wil, +1, (const double2 *)X, ldx, (double2 *)ctx->T, ctx->ldv, ncols, mask, ctx->cs);
-  launch_wilson_dslash(ctx->wil, -1, (const double2 *)ctx->T, ctx->ldv, (double2 *)Y, ldy, ncols, mask, ctx->cs);
-  return 2;
+  const int64_t ld = ctx->ldv;
+  if (!ctx->links_ready || !fix_pays(ctx, ncols)) {   // (a call that prepared no fixed-point form does without)
+    launch_wilson_dslash(ctx->wil, +1, (const double2 *)X, ldx, (double2 *)ctx->T, ld, ncols, mask, ctx->cs);
+    launch_wilson_dslash(ctx->wil, -1, (const double2 *)ctx->T, ld, (double2 *)Y, ldy, ncols, mask, ctx->cs);
+    return 2;
+  }
+  launch_fix_spinors(ctx->wfix, (const double2 *)X, ldx, ctx->F, ld, ctx->Fe, ncols, mask, ctx->cs);
+  launch_dslash_fix(ctx->wfix, +1, ctx->F, ctx->Fe, ld, fix_T(ctx), fix_Te(ctx), nullptr, 0, ncols, mask, ctx->cs);
+  launch_dslash_fix(ctx->wfix, -1, fix_T(ctx), fix_Te(ctx), ld, nullptr, nullptr, (double2 *)Y, ldy, ncols, mask,
+                    ctx->cs);
+  return 3;
 }
 
 // Y = A X with the FP32 copy of the operator (mixed precision).  Returns the kernel count.
@@ -446,7 +502,7 @@ int issue_seed_step(seed_ctx *ctx, int nrhs, bool reorth) {
   SeedBufs<T> b = seed_bufs<T>(ctx, nrhs);
   // u = A f with f = beta_{i-1} v_i not yet normalized: the dots kernel forms v_i and scales u
   int k = kLow<T> ? apply_A32(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1, nullptr)
-                  : apply_A(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1, nullptr);
+                  : apply_A64(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1);
   launch_seed_dots<T>(b, ctx->cs);
   launch_seed_update<T>(b, !reorth, ctx->cs);
   k += 2;
@@ -670,6 +726,7 @@ seed_status solve_first_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
   const int64_t n = ctx->n;
   const seed_params &p = ctx->prm;
   TRY(ensure_cols(ctx, std::max(nrhs, 1)));
+  TRY(ensure_fixed(ctx));
   if (blocked_seeding(ctx, nrhs)) TRY(ensure_block(ctx));
   ctx->basis_valid = false;
   ctx->seeded = false;
@@ -697,7 +754,7 @@ seed_status solve_first_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
     if (nrhs > 1) launch_copy_cols<T>((const T *)B + ldb, ldb, (T *)ctx->R, ctx->ldv, n, nrhs - 1, ctx->cs);
     kern += 1 + (nrhs > 1);
   } else {
-    kern += apply_A(ctx, X, ldx, ctx->Q, ctx->ldv, nrhs, nullptr);
+    kern += apply_A64(ctx, X, ldx, ctx->Q, ctx->ldv, nrhs);
     ctx->stats.mvps += nrhs;
     launch_sub_from<T>((const T *)B, ldb, (const T *)ctx->Q, ctx->ldv, (T *)ctx->P, ctx->ldv, n, nrhs, ctx->cs);
     if (nrhs > 1) launch_copy_cols<T>((const T *)ctx->P + ctx->ldv, ctx->ldv, (T *)ctx->R, ctx->ldv, n, nrhs - 1, ctx->cs);
@@ -770,20 +827,23 @@ int issue_cg_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, const 
                   unsigned *tickets) {
   const int64_t n = ctx->n, ld = ctx->ldv;
   T *P = (T *)ctx->P + (int64_t)c0 * ld, *Q = (T *)ctx->Q + (int64_t)c0 * ld, *R = (T *)ctx->R + (int64_t)c0 * ld;
-  int k;
-  if (ctx->kind == 0) {
-    launch_csr_spmv(ctx->csr, (const double *)P, ld, (double *)Q, ld, c.nc, c.active, s);
-    k = 1;
+  if constexpr (std::is_same_v<T, double2>) {
+    // p's blocks are in F: t = D p, q = D^H t with alpha, the residual, then x and p (with its blocks)
+    int4 *Fb = ctx->F + (int64_t)c0 * ld, *Tb = fix_T(ctx) + (int64_t)c0 * ld;
+    int32_t *Fe = ctx->Fe + (int64_t)c0 * (ld / 12), *Te = fix_Te(ctx) + (int64_t)c0 * (ld / 12);
+    const FixDot dot{P, ctx->dotpart + (int64_t)c0 * (ld / 192), tickets, c.rho, c.alpha};
+    launch_dslash_fix(ctx->wfix, +1, Fb, Fe, ld, Tb, Te, nullptr, 0, c.nc, c.active, s);
+    launch_dslash_fix(ctx->wfix, -1, Tb, Te, ld, nullptr, nullptr, Q, ld, c.nc, c.active, s, &dot);
+    launch_cg_residual(n, R, Q, ld, c, partials, tickets, s);
+    launch_cg_xp_fix(ctx->wfix, call, R, P, ld, Fb, Fe, c, s);
+    return 4;
   } else {
-    double2 *Tb = (double2 *)ctx->T + (int64_t)c0 * ld;
-    launch_wilson_dslash(ctx->wil, +1, (const double2 *)P, ld, Tb, ld, c.nc, c.active, s);
-    launch_wilson_dslash(ctx->wil, -1, Tb, ld, (double2 *)Q, ld, c.nc, c.active, s);
-    k = 2;
+    launch_csr_spmv(ctx->csr, P, ld, Q, ld, c.nc, c.active, s);
+    launch_cg_alpha<T>(n, P, Q, ld, c, partials, tickets, s);
+    launch_cg_update<T>(n, call, R, P, Q, ld, c, partials, tickets, s);
+    launch_cg_p<T>(n, R, P, ld, c, s);
+    return 4;
   }
-  launch_cg_alpha<T>(n, P, Q, ld, c, partials, tickets, s);
-  launch_cg_update<T>(n, call, R, P, Q, ld, c, partials, tickets, s);
-  launch_cg_p<T>(n, R, P, ld, c, s);
-  return k + 3;
 }
 
 // The columns c0 .. c0 + nc - 1 of the per-column CG state.
@@ -802,20 +862,27 @@ CgCols cg_sub(const CgCols &c, int c0, int nc) {
 // the others' operator applies.  Branch b owns columns start[b] .. start[b+1]-1,
 // CallArgs slot b, the b-th part of the partials and the tickets shifted by
 // start[b].
-int cg_branches(int nc, int start[kCgBranches + 1]) {
+int cg_branches(int nc, int start[kCgBranches + 1], int most = kCgBranches) {
   int nb = nc / 2;
-  if (nb > kCgBranches) nb = kCgBranches;
+  if (nb > most) nb = most;
   if (nb < 1) nb = 1;
   for (int b = 0; b <= nb; ++b) start[b] = b * nc / nb;
   return nb;
 }
 
+// Branches of the FP64 CG graphs: all, except for the Wilson operator on few tiles x columns, where
+// every launch is one short wave and three branches only contend for launch slots
+// (4^4 x 11 columns 4.68 -> 4.48 ms; 8^4 x 11 columns 11.5 ms with one branch, 10.0 with three).
+int cg_most(const seed_ctx *ctx, int nc) {
+  return ctx->kind == 1 && ctx->precision == 0 && fix_few(ctx->wfix.sites, nc) ? 1 : kCgBranches;
+}
+
 // Captures `len` iterations of issue(view, first column, stream, branch) on
 // every branch: a fork from cs, the branches, a join back into cs.
 template <class F>
-int issue_cg_branches(seed_ctx *ctx, const CgCols &c, int len, F &&issue) {
+int issue_cg_branches(seed_ctx *ctx, const CgCols &c, int len, int most, F &&issue) {
   int start[kCgBranches + 1];
-  const int nb = cg_branches(c.nc, start);
+  const int nb = cg_branches(c.nc, start, most);
   int k = 0;
   if (nb > 1) {
     cudaEventRecord(ctx->ev_fork, ctx->cs);   // a failed call invalidates the capture (reported at its end)
@@ -891,7 +958,7 @@ seed_status launch_cg_run(seed_ctx *ctx, const CgCols &c, int len) {
     GraphEntry g;
     cudaGraph_t graph;
     CU(cudaStreamBeginCapture(ctx->cs, cudaStreamCaptureModeThreadLocal));
-    g.kernels += issue_cg_branches(ctx, c, len, [&](const CgCols &v, int c0, cudaStream_t s, int b) {
+    g.kernels += issue_cg_branches(ctx, c, len, cg_most(ctx, c.nc), [&](const CgCols &v, int c0, cudaStream_t s, int b) {
       return issue_cg_iter<T>(ctx, v, c0, s, ctx->call + b, branch_partials(ctx, b), ctx->tickets + c0);
     });
     CU(cudaStreamEndCapture(ctx->cs, &graph));
@@ -917,21 +984,28 @@ seed_status cg_impl(seed_ctx *ctx, const T *Bc, int64_t ldb, T *Xc, int64_t ldx,
   CU(cudaEventRecord(ctx->t2, ctx->cs));
   // slot b: branch b of the CG graphs (its first column)
   int start[kCgBranches + 1];
-  const int nb = cg_branches(nc, start);
+  const int nb = cg_branches(nc, start, cg_most(ctx, nc));
   CallArgs ca[kCgBranches];
   for (int b = 0; b < nb; ++b) ca[b] = CallArgs{Xc, ldx, start[b]};
   CU(cudaMemcpyAsync(ctx->call, ca, sizeof(CallArgs) * nb, cudaMemcpyHostToDevice, ctx->cs));
   const CgCols c = cg_cols(ctx, nc);
+  TRY(ensure_fixed(ctx));
   // K7: true residual of the seeded systems, then p = r
   int kern = apply_A(ctx, Xc, ldx, ctx->Q, ld, nc, nullptr);
   launch_cg_init<T>(n, Bc, ldb, (const T *)ctx->Q, ld, (T *)ctx->R, (T *)ctx->P, ld, c, ctx->partials, ctx->tickets,
                     false, ctx->cs);
   ctx->stats.kernel_launches += kern + 1;
   ctx->stats.mvps += nc;
-
   ReorthRun scg;   // small real CSR problems: the one-launch CG with two barriers per iteration
   if constexpr (std::is_same_v<T, double>) scg = small_cg_shape(ctx, nc);
   const bool persist = scg.grid > 0 || (ctx->allow_persistent_cg && ctx->pgrid_cg > 0 && nc <= kPersistMaxCols);
+  auto blocks_of_p = [&]() {   // Wilson: p's fixed-point blocks, kept up by the iterations from here on
+    if (ctx->kind != 1 || persist) return;
+    launch_fix_spinors(ctx->wfix, (const double2 *)ctx->P, ld, ctx->F, ld, ctx->Fe, nc, c.active, ctx->cs);
+    ctx->stats.kernel_launches += 1;
+  };
+  blocks_of_p();
+
   const GridSync g = grid_sync_bufs(ctx);
   const int L = 16;
   for (int round = 0;; ++round) {
@@ -985,6 +1059,7 @@ seed_status cg_impl(seed_ctx *ctx, const T *Bc, int64_t ldb, T *Xc, int64_t ldx,
     launch_cg_check<T>(n, Bc, ldb, (const T *)ctx->Q, ld, (T *)ctx->R, ld, c, ctx->partials, ctx->tickets, ctx->cs);
     launch_cg_init<T>(n, Bc, ldb, (const T *)ctx->Q, ld, (T *)ctx->R, (T *)ctx->P, ld, c, ctx->partials,
                       ctx->tickets, true, ctx->cs);
+    blocks_of_p();
     ctx->stats.kernel_launches += kern + 2;
     CU(cudaMemcpyAsync(ctx->h_flags, c.active, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost, ctx->cs));
     CU(cudaStreamSynchronize(ctx->cs));
@@ -1125,6 +1200,7 @@ seed_status solve_related_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *
   if (info && nc > 0) std::memset(info + 1, 0, sizeof(seed_info) * nc);
   if (nc <= 0) return SEED_OK;
   TRY(ensure_cols(ctx, nrhs));
+  TRY(ensure_fixed(ctx));
   TRY(ensure_related(ctx, nc));
   const T *Bt = (const T *)B;
   T *Xt = (T *)X;
@@ -1201,6 +1277,7 @@ seed_status solve_multiple_impl(seed_ctx *ctx, const void *B, int64_t ldb, void 
   c.max_restarts = 0;
   c.tol_check = 1.5 * c.tol;
   const int L = 16;
+  TRY(ensure_fixed(ctx));
   for (int j = 0; j < nrhs; ++j) {
     const CallArgs ca{Xw, ld, j};
     CU(cudaMemcpyAsync(ctx->call, &ca, sizeof(ca), cudaMemcpyHostToDevice, ctx->cs));
@@ -1353,7 +1430,7 @@ seed_status mixed_cg(seed_ctx *ctx, const T64 *Bc, int64_t ldb, T64 *Xc, int64_t
   cudaEvent_t evs[2] = {nullptr, nullptr};
   for (;;) {
     TRY(run_graph(ctx, key, [&] {
-      return issue_cg_branches(ctx, c, L, [&](const CgCols &v, int cb0, cudaStream_t s, int b) {
+      return issue_cg_branches(ctx, c, L, kCgBranches, [&](const CgCols &v, int cb0, cudaStream_t s, int b) {
         return issue_mixed_iter<T32>(ctx, v, cb0, s, ctx->call32 + 1 + b, branch_partials(ctx, b), ctx->tickets + cb0);
       });
     }));
@@ -1394,6 +1471,7 @@ seed_status solve_first_mixed(seed_ctx *ctx, const void *B, int64_t ldb, void *X
   const int64_t n = ctx->n, ld = ctx->ldv;
   const seed_params &p = ctx->prm;
   TRY(ensure_cols(ctx, std::max(nrhs, 1)));
+  TRY(ensure_fixed(ctx));
   if (blocked_seeding(ctx, nrhs)) TRY(ensure_block(ctx));
   ctx->basis_valid = false;
   ctx->seeded = false;
@@ -1506,6 +1584,7 @@ seed_status solve_rest_mixed(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
   if (info) std::memset(info + 1, 0, sizeof(seed_info) * (nc > 0 ? nc : 0));
   if (nc <= 0) return SEED_OK;
   TRY(ensure_cols(ctx, nrhs));
+  TRY(ensure_fixed(ctx));
   CU(cudaEventRecord(ctx->t2, ctx->cs));
   TRY((mixed_cg<T64, T32>(ctx, (const T64 *)B + ldb, ldb, (T64 *)X + ldx, ldx, 1, nc, ctx->prm.tol_rest, nullptr)));
   CU(cudaEventRecord(ctx->t3, ctx->cs));
@@ -1554,6 +1633,7 @@ bool overlap(const void *a, int64_t lda, const void *b, int64_t ldb, int cols, i
 struct StreamScope {
   seed_ctx *ctx;
   explicit StreamScope(seed_ctx *c) : ctx(c) {
+    ctx->links_ready = false;   // ensure_fixed
     if (ctx->in_batch) return;
     cudaEventRecord(ctx->ev_in, ctx->user_stream);
     cudaStreamWaitEvent(ctx->cs, ctx->ev_in, 0);
@@ -1594,6 +1674,7 @@ seed_status create_common(seed_ctx *ctx, const seed_params *p, seed_stream strea
 void destroy(seed_ctx *ctx) {
   if (!ctx) return;
   if (ctx->cs) cudaStreamSynchronize(ctx->cs);
+  cudaFree(ctx->flinks); cudaFree(ctx->fexp); cudaFree(ctx->F); cudaFree(ctx->Fe); cudaFree(ctx->dotpart);
   for (auto &kv : ctx->graphs) cudaGraphExecDestroy(kv.second.exec);
   void *ptrs[] = {ctx->V, ctx->u, ctx->f, ctx->w, ctx->st, ctx->alpha_hist, ctx->beta_hist,
                   ctx->delta_hist, ctx->eta, ctx->partials, ctx->tickets, ctx->Hpart, ctx->H, ctx->call,
@@ -1732,6 +1813,8 @@ seed_status seed_create_wilson(seed_ctx **out, const seed_wilson *A, const seed_
   ctx->nv = ctx->lay.length(ctx->n);
   s = alloc_common(ctx);
   if (s == SEED_OK) s = dalloc(ctx, &ctx->nbr, sizeof(int32_t) * 8 * vol);
+  if (s == SEED_OK) s = dalloc(ctx, &ctx->flinks, sizeof(int4) * 4 * 288 * (size_t)((vol + 31) / 32));
+  if (s == SEED_OK) s = dalloc(ctx, &ctx->fexp, sizeof(int32_t) * 4 * vol);
   if (s == SEED_OK && ctx->precision == 1) {
     const int64_t nl = 4 * vol * 9;
     s = dalloc(ctx, &ctx->op32, sizeof(float2) * (size_t)nl);
@@ -1749,6 +1832,14 @@ seed_status seed_create_wilson(seed_ctx **out, const seed_wilson *A, const seed_
     ctx->wil.bc_t = A->bc_t;
     ctx->wil.links = (const double2 *)A->links;
     ctx->wil.nbr = ctx->nbr;
+    for (int k = 0; k < 4; ++k) ctx->wfix.dims[k] = A->dims[k];
+    ctx->wfix.sites = vol;
+    ctx->wfix.kappa = A->kappa;
+    ctx->wfix.bc_t = A->bc_t;
+    ctx->wfix.links = (const double2 *)A->links;
+    ctx->wfix.nbr = ctx->nbr;
+    ctx->wfix.flinks = ctx->flinks;
+    ctx->wfix.fexp = ctx->fexp;
     for (int k = 0; k < 4; ++k) ctx->wil32.dims[k] = A->dims[k];
     ctx->wil32.sites = vol;
     ctx->wil32.kappa = A->kappa;
@@ -1801,6 +1892,7 @@ seed_status seed_solve_cg(seed_ctx *ctx, const void *B, int64_t ldb, void *X, in
   if (overlap(B, ldb, X, ldx, ncols, ctx->n, ctx->esz)) return fail(ctx, SEED_EINVAL, "B and X overlap");
   StreamScope scope(ctx);
   TRY(ensure_cols(ctx, ncols));
+  TRY(ensure_fixed(ctx));
   if (ctx->precision == 1) {
     if (info) std::memset(info, 0, sizeof(seed_info) * ncols);
     CU(cudaEventRecord(ctx->t2, ctx->cs));
@@ -1891,6 +1983,7 @@ seed_status seed_project(seed_ctx *ctx, const void *B, int64_t ldb, void *X, int
   if (overlap(B, ldb, X, ldx, ncols, ctx->n, ctx->esz)) return fail(ctx, SEED_EINVAL, "B and X overlap");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
+  if (!ctx->prm.x0_zero) TRY(ensure_fixed(ctx));
   const int64_t n = ctx->n, ld = ctx->ldv;
   int kern = 0;
   if (ctx->kind == 0) {
@@ -1943,6 +2036,7 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   if (overlap(X, ldx, Y, ldy, ncols, len, es)) return fail(ctx, SEED_EINVAL, "X and Y overlap");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
+  if (op == 0 && fix_pays(ctx, ncols)) TRY(ensure_fixed(ctx));
   if (op == 3) {
     ctx->stats.kernel_launches += apply_A32(ctx, X, ldx, Y, ldy, ncols, nullptr, false);
   } else if (op >= 4) {
@@ -1953,6 +2047,7 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
     ctx->stats.kernel_launches += apply_A(ctx, X, ldx, Y, ldy, ncols, nullptr);
     ctx->stats.mvps += ncols;
   } else {
+    // D and D^H by themselves form right-hand sides of the seed system (b = D^H eta): FP64, see apply_A64
     launch_wilson_dslash(ctx->wil, op == 1 ? +1 : -1, (const double2 *)X, ldx, (double2 *)Y, ldy, ncols, nullptr,
                          ctx->cs);
     ctx->stats.kernel_launches += 1;
@@ -2051,6 +2146,7 @@ seed_status seed_time_operator(seed_ctx *ctx, int32_t op, int32_t ncols, int32_t
   if (ncols < 1 || ncols > kMaxRhs || reps < 1 || reps > 100000) return fail(ctx, SEED_EINVAL, "bad ncols / reps");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
+  if (op == 0 && fix_pays(ctx, ncols)) TRY(ensure_fixed(ctx));
   CU(cudaMemsetAsync(ctx->P, 0x3F, (size_t)ctx->ldv * ncols * ctx->esz, ctx->cs));   // normal doubles ~4.8e-4
   if (op >= 3) CU(cudaMemsetAsync(ctx->P32, 0x3F, (size_t)ctx->ldv * ncols * ctx->vsz, ctx->cs));   // floats ~0.75
   // one untimed launch, then the timed ones

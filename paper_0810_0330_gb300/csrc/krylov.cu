@@ -886,6 +886,38 @@ __global__ void __launch_bounds__(NT) k_cg_update(int64_t n, const CallArgs *cal
   if (threadIdx.x == 0) cg_update_tail(c, col, rr);
 }
 
+// The same without x, which launch_cg_xp_fix (wilson_fixed.cu) updates with p;
+// upd[col] tells it which columns did an iteration.
+__global__ void __launch_bounds__(NT) k_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, CgCols c,
+                                                    double *partials, unsigned *tickets) {
+  __shared__ double sm[NT / 32];
+  const int col = blockIdx.y;
+  if (!c.active[col]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) c.upd[col] = 0;
+    return;
+  }
+  R += (int64_t)col * ld;
+  Q += (int64_t)col * ld;
+  const double a = c.alpha[col];
+  double acc = 0.0;
+#pragma unroll 4
+  GRID_STRIDE(e, n) {
+    const double2 r = Sc<double2>::axpy(-a, Q[e], R[e]);
+    R[e] = r;
+    acc = Sc<double2>::nrm2(r, acc);
+  }
+  double v[1] = {acc};
+  block_sum<1, NT>(v, sm);
+  double *part = partials + (int64_t)col * gridDim.x;
+  if (threadIdx.x == 0) part[blockIdx.x] = v[0];
+  if (!last_block_done(tickets + kColTicket + col, gridDim.x)) return;
+  const double rr = sum_partials<NT>(part, gridDim.x, 1, 0, sm);
+  if (threadIdx.x == 0) {
+    c.upd[col] = 1;
+    cg_update_tail(c, col, rr);
+  }
+}
+
 // p = r + beta p (also used with beta = 0 after a restart: p = r)
 template <class T>
 __global__ void __launch_bounds__(NT) k_cg_p(int64_t n, const T *R, T *P, int64_t ld, CgCols c, int copy_only) {
@@ -959,6 +991,11 @@ void launch_cg_update(int64_t n, const CallArgs *call, T *R, const T *P, const T
                       double *partials, unsigned *tickets, cudaStream_t s) {
   dim3 g((unsigned)col_blocks(n, c.nc), (unsigned)c.nc);
   k_cg_update<T><<<g, NT, 0, s>>>(n, call, R, P, Q, ld, c, partials, tickets);
+}
+void launch_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, const CgCols &c, double *partials,
+                        unsigned *tickets, cudaStream_t s) {
+  dim3 g((unsigned)col_blocks(n, c.nc), (unsigned)c.nc);
+  k_cg_residual<<<g, NT, 0, s>>>(n, R, Q, ld, c, partials, tickets);
 }
 template <class T>
 void launch_cg_p(int64_t n, const T *R, T *P, int64_t ld, const CgCols &c, cudaStream_t s) {

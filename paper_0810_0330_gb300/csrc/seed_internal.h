@@ -191,6 +191,38 @@ void launch_wilson_dslash32(const WilsonOp32 &op, int sign, const float2 *in, in
                             int ncols, const int32_t *col_active, bool tiled, cudaStream_t s);
 void launch_links_soa32(const double2 *links, float2 *out, int64_t sites, cudaStream_t s);
 
+// The FP64 operator in fixed-point arithmetic (wilson_fixed.cuh): WilsonOp plus
+// the fixed-point copy of -kappa U.  Spinor vectors: limbs q (columns ldq
+// elements apart, ldq = 384 * tiles) and site exponents e (ldq / 12 apart).
+struct WilsonFix {
+  int32_t dims[4];
+  int64_t sites;
+  double kappa;
+  int32_t bc_t;
+  const double2 *links;   // the caller's links
+  const int32_t *nbr;
+  const int4 *flinks;     // [4][tiles][9][32] limbs
+  const int32_t *fexp;    // [4][sites] exponents
+};
+void launch_fix_links(const WilsonFix &op, cudaStream_t s);   // fills flinks and fexp from links
+void launch_fix_spinors(const WilsonFix &op, const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e,
+                        int ncols, const int32_t *col_active, cudaStream_t s);
+// few enough tiles x columns for the form with one warp per direction and half-spinor component
+bool fix_few(int64_t sites, int ncols);
+// lockstep CG's alpha[col] = rho[col] / Re(P^H out), formed with the last operator half
+// (P: ldo apart; part: ceil(sites / 16) doubles per column; tickets as CgCols' reductions)
+struct FixDot {
+  const double2 *P;
+  double *part;
+  unsigned *tickets;
+  const double *rho;
+  double *alpha;
+};
+// (q, e) -> (qout, eout), or -> out (doubles, site-major, ldo) when qout is NULL; dot: with D^H only
+void launch_dslash_fix(const WilsonFix &op, int sign, const int4 *in, const int32_t *ein, int64_t ldq, int4 *qout,
+                       int32_t *eout, double2 *out, int64_t ldo, int ncols, const int32_t *col_active,
+                       cudaStream_t s, const FixDot *dot = nullptr);
+
 // CSR (csr.cu)
 template <class R>
 struct CsrOpT {
@@ -231,6 +263,12 @@ template <class T> void launch_cg_alpha(int64_t n, const T *P, const T *Q, int64
                                         double *partials, unsigned *tickets, cudaStream_t s);
 template <class T> void launch_cg_update(int64_t n, const CallArgs *call, T *R, const T *P, const T *Q, int64_t ld,
                                          const CgCols &c, double *partials, unsigned *tickets, cudaStream_t s);
+// The Wilson CG's form: r and its norm only (X untouched), sets upd[col] for launch_cg_xp_fix
+void launch_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, const CgCols &c, double *partials,
+                        unsigned *tickets, cudaStream_t s);
+// x += alpha p, p = r + beta p and p's blocks (q, e), columns with upd set
+void launch_cg_xp_fix(const WilsonFix &op, const CallArgs *call, const double2 *R, double2 *P, int64_t ld, int4 *q,
+                      int32_t *e, const CgCols &c, cudaStream_t s);
 template <class T> void launch_cg_p(int64_t n, const T *R, T *P, int64_t ld, const CgCols &c, cudaStream_t s);
 template <class T> void launch_cg_check(int64_t n, const T *B, int64_t ldb, const T *Q, int64_t ldq, T *R,
                                         int64_t ld, const CgCols &c, double *partials, unsigned *tickets,
