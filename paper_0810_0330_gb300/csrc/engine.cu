@@ -108,8 +108,8 @@ struct seed_ctx {
   int32_t *h_gerr = nullptr;           // pinned copy of the error flag
   void *f2 = nullptr;                  // second Lanczos-vector buffer (CSR persistent run)
   double *tpart = nullptr;             // per-tile partial sums (persistent Wilson seed run)
-  int rgrid_cap[2] = {0, 0};           // most blocks of a reorthogonalizing CSR run, 16 / 32 rows per block
-  int scg_cap[2] = {0, 0};             // most blocks of the small-problem CSR CG, 16 / 32 rows per block
+  int rgrid_cap[3] = {0, 0, 0};        // most blocks of a reorthogonalizing CSR run, 16 / 32 / 64 rows per block
+  int scg_cap[3] = {0, 0, 0};          // most blocks of the small-problem CSR CG, 16 / 32 / 64 rows per block
   bool allow_small_cg = true;          // the small-problem CSR CG (not on kernel_path 1)
   double *rhpart = nullptr;            // its partial products, 2 x (m_max + 1) x grid doubles
   double2 *Hrows = nullptr;            // FP32 reorthogonalization partials by 4096-row chunks (long vectors)
@@ -284,7 +284,7 @@ seed_status alloc_common(seed_ctx *ctx) {
   ctx->pgrid = coop ? persistent_grid(ctx->kind, ctx->sm_count, false, ctx->precision == 1) : 0;
   ctx->pgrid_cg = coop ? persistent_grid(ctx->kind, ctx->sm_count, true) : 0;
   if (coop && ctx->kind == 0 && ctx->precision == 0)
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < 3; ++q) {
       ctx->rgrid_cap[q] = reorth_run_grid_cap(ctx->sm_count, 16 << q);
       ctx->scg_cap[q] = small_cg_grid_cap(ctx->sm_count, 16 << q);
     }
@@ -574,46 +574,37 @@ int cg_csr_grid(const seed_ctx *ctx, int nc) {
   return (int)std::min<int64_t>(ctx->pgrid_cg, std::max<int64_t>(1, items));
 }
 
-// The one-launch seed run of small real CSR problems that reorthogonalize every
-// 1 to 7 steps (the streaming form of the seeding): rows per block (16, or 32
-// when 16 would need more blocks than can be resident) and the grid; grid 0
-// when the problem does not qualify.
+// The one-launch seed run and lockstep CG of small real CSR problems: rows per
+// block, the smallest of 16, 32, 64 whose grid has no more blocks than there are
+// SMs (a barrier of 256 blocks takes 4.2 us, of 128 blocks 3.1 us) or, failing that,
+// than can be resident; grid 0 when the problem does not qualify.
 struct ReorthRun {
   int rb = 0, grid = 0;
 };
-ReorthRun reorth_run_shape(const seed_ctx *ctx, int nrhs) {
-  const int f = ctx->prm.reorth_freq;
+ReorthRun small_run_shape(const seed_ctx *ctx, const int (&cap)[3]) {
   ReorthRun r;
-  if (!ctx->allow_persistent || ctx->kind != 0 || ctx->precision != 0 || f < 1 || f >= 8) return r;
-  if (nrhs > kReorthRunMaxRhs || ctx->n > kReorthRunMaxN || ctx->n < 1) return r;
-  for (int q = 0; q < 2; ++q) {
-    const int rb = 16 << q;
-    const int64_t grid = (ctx->n + rb - 1) / rb;
-    if (grid <= ctx->rgrid_cap[q]) {
-      r.rb = rb;
-      r.grid = (int)grid;
-      return r;
+  if (ctx->n > kReorthRunMaxN || ctx->n < 1) return r;
+  for (int blocks_per_sm = 1; blocks_per_sm <= 2; ++blocks_per_sm)
+    for (int q = 0; q < 3; ++q) {
+      const int64_t grid = (ctx->n + (16 << q) - 1) / (16 << q);
+      if (grid <= cap[q] && grid <= (int64_t)blocks_per_sm * ctx->sm_count) {
+        r.rb = 16 << q;
+        r.grid = (int)grid;
+        return r;
+      }
     }
-  }
   return r;
 }
-
-// The one-launch lockstep CG of small real CSR problems: rows per block and
-// grid, as for the reorthogonalizing seed run; grid 0 when it does not apply.
+// the seed run, when it reorthogonalizes every 1 to 7 steps (the streaming form of the seeding)
+ReorthRun reorth_run_shape(const seed_ctx *ctx, int nrhs) {
+  const int f = ctx->prm.reorth_freq;
+  if (!ctx->allow_persistent || ctx->kind != 0 || ctx->precision != 0 || f < 1 || f >= 8) return {};
+  return nrhs > kReorthRunMaxRhs ? ReorthRun{} : small_run_shape(ctx, ctx->rgrid_cap);
+}
+// the lockstep CG
 ReorthRun small_cg_shape(const seed_ctx *ctx, int nc) {
-  ReorthRun r;
-  if (!ctx->allow_small_cg || ctx->kind != 0 || ctx->precision != 0 || nc > 16 || nc < 1) return r;
-  if (ctx->n > kReorthRunMaxN || ctx->n < 1) return r;
-  for (int q = 0; q < 2; ++q) {
-    const int rb = 16 << q;
-    const int64_t grid = (ctx->n + rb - 1) / rb;
-    if (grid <= ctx->scg_cap[q]) {
-      r.rb = rb;
-      r.grid = (int)grid;
-      return r;
-    }
-  }
-  return r;
+  if (!ctx->allow_small_cg || ctx->kind != 0 || ctx->precision != 0 || nc > 16 || nc < 1) return {};
+  return small_run_shape(ctx, ctx->scg_cap);
 }
 
 seed_status seed_reorth_run(seed_ctx *ctx, int nrhs, ReorthRun shape) {

@@ -79,6 +79,26 @@ SEED_DEV bool grid_sync(const GridSync &g, unsigned &epoch) {
   return s_ok != 0;
 }
 
+// the two halves of grid_sync: work between them overlaps the wait (thread 0 polls
+// in the second); both contain CTA barriers
+SEED_DEV void grid_arrive(const GridSync &g, unsigned &epoch) {
+  __syncthreads();
+  ++epoch;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(g.count, 1u);
+  }
+}
+SEED_DEV bool grid_wait(const GridSync &g, unsigned epoch) {
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
+    s_ok = wait_geq(g.count, epoch * gridDim.x, g.error) ? 1 : 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 template <class F>
 SEED_DEV bool grid_reduce_sync(const GridSync &g, unsigned &epoch, F &&last_block_work) {
   __shared__ int s_last, s_ok;
@@ -1263,137 +1283,275 @@ __global__ void __launch_bounds__(PT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> op
 // g^j = v_i^H r_0^j, the LU update with x^1 += zeta_i w_i and
 // x^j += eta^j w_i, and on reorthogonalizing steps the classical Gram-Schmidt
 // passes over V_{<i}, the renormalization of v_i and the projections of f on
-// it -- in one cooperative launch, instead of 10 to 14 kernels per step.
+// it -- in one cooperative launch.
 //
-// Block b owns rows [b RB, (b + 1) RB) (RB = 16 or 32, so that the grid spans
-// most SMs even for n = 4096); thread t < RB holds row b RB + t in every row
-// phase.  The products with V_{<i} run with one thread per basis column
-// (columns t, t + PT, ...): a thread loads its column's RB rows (one or two
-// 128-byte lines), so the whole grid streams V with many loads in flight.
-//   H = V_{<i}^H [v_i f]: per block and column the dot products over the
-//   block's rows, written to hpart[(2 c + v) G + b]; after a barrier block b
-//   sums the values [2 k b / G, 2 k (b + 1) / G) over the blocks in block order
-//   into H; after a second barrier each thread adds x_rc H_c of its columns
-//   into 2 RB row sums, the block combines them (warp reduce-scatter, then the
-//   warps in order), and the rows subtract them.  When a second pass follows,
-//   its dot products use the same lines again (from L1) in the same phase.
-// Scalar sums (alpha_i with the g^j, ||v_i||^2, v_i^H f, ||f||^2): one row of
-// block partials per block in one of two alternating regions -- a block that
-// has run ahead writes the other region while slower blocks still read this
-// one -- reduced by every block in block order, so the blocks' shared-memory
-// copies of the recurrence's scalars stay identical.
+// What a step costs here is grid barriers (3.1 us with the sums after it at 128 blocks, 4.2
+// at 256) and FP64 operations, so there are few of both:
+//  - one block per SM at most: block b owns rows [b RB, (b + 1) RB), RB the smallest
+//    of 16, 32, 64 that needs no more blocks than SMs;
+//  - five barriers per reorthogonalizing step (two passes).  The products of the first pass
+//    are formed with u = A v_i - beta_{i-1} v_{i-1} before alpha_i is known:
+//    V^H f = V^H u - alpha_i V^H v_i, one barrier for both.  ||v_i||^2 and v_i^H f
+//    of the normalization come with the second pass's products: that pass changes them by
+//    the square of its coefficients, below rounding.  The last projection's
+//    coefficient h and ||f||^2 come together, and f - h v_i is formed by whoever reads f next;
+//  - a block's rows of V stay in shared memory, as 57-bit integers in two limbs
+//    (|V| <= 1), and the products with them are integer multiply-adds
+//    (wilson_fixed.cuh has the rates): per block and column exact sums of products cut off 2^-55
+//    below the block's largest factor, which is below the rounding errors of the
+//    FP64 sums they replace.  Columns past kcap (shared memory) are read from V in FP64.
+//   H = V_{<i}^H [v_i u]: per block and column the sums over the block's rows,
+//   written to hpart[(2 c + v) G + b]; after a barrier block b sums the values [2 k b /
+//   G, 2 k (b + 1) / G) over the blocks in block order into H; after a second
+//   barrier the rows subtract V H.
+// Scalar sums (alpha_i with the g^j, the norms): one row of block partials per
+// block in one of two alternating regions -- a block that has run ahead writes
+// the other region while slower blocks still read this one -- reduced by every
+// block in block order, so the blocks' shared-memory copies of the recurrence's
+// scalars stay identical.
+// 64 x 64 Laplacian, 251 steps, reorthogonalizing every step: 12.9 -> 6.4 ms (256
+// blocks of 128 threads, eight barriers a step, V from L2, FP64 products before).
 // ---------------------------------------------------------------------------
 constexpr int kRunRegion = 32;                 // doubles per block in a scalar partial region
 constexpr int kRunMaxRhs = kReorthRunMaxRhs;   // alpha_i and g^2..g^16 in one region row
-
-// block sums of v[0..nv) into row[0..nv) (warp sums, then the four warps in order)
-template <int NV>
-SEED_DEV void block_row(const double (&v)[NV], int nv, double *row, double (*s)[kRunRegion]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    if (q < nv) {
-      const double t = warp_sum(v[q]);
-      if (lane == 0) s[warp][q] = t;
-    }
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < nv)
-    row[threadIdx.x] = ((s[0][threadIdx.x] + s[1][threadIdx.x]) + s[2][threadIdx.x]) + s[3][threadIdx.x];
-}
+constexpr int RT = 256;                        // threads per block
+constexpr int kRunSmem = 100 * 1024;           // shared memory of V's rows and H: two problems' blocks fit an SM
+constexpr int kVBits = 57, kYBits = 55, kHBits = 51;   // V, the block's v_i / u / f, H: |I| < 2^bits
 
 // after the barrier: S[q] = sum over blocks (in block order) of region[b * kRunRegion + q], q < nv
 SEED_DEV void reduce_region(const double *region, int nv, double *S) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int q = warp; q < nv; q += PT / 32) {
+  for (int q = warp; q < nv; q += blockDim.x / 32) {
     const double t = warp_sum_partials(region, gridDim.x, kRunRegion, q);
     if (lane == 0) S[q] = t;
   }
   __syncthreads();
 }
 
-// hpart[(2 c + v) G + b] = sum over the block's rows r of V[c][row0 + r] y_v[r], c < k
-template <int RB>
-SEED_DEV void col_dots(const double *V, int64_t ldv, int64_t row0, int rows, int k, const double (*y)[RB],
-                       double *hpart) {
-  const int G = gridDim.x;
-  for (int c = threadIdx.x; c < k; c += PT) {
-    const double *vc = V + (int64_t)c * ldv + row0;
-    double x[RB];
+// One warp: the sum of p[0], p[stride], ... (nb values) with as few dependent FP64 adds
+// as there are (each occupies its sub-partition's FP64 unit for 64 clocks); fixed order.
+SEED_DEV double warp_sum_few(const double *p, int nb, int stride) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int b0 = 0; b0 < nb; b0 += 256) {
+    double v[8];
 #pragma unroll
-    for (int r = 0; r < RB; ++r) x[r] = r < rows ? vc[r] : 0.0;
-    double hv = 0.0, hf = 0.0;
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      hv = fma(x[r], y[0][r], hv);
-      hf = fma(x[r], y[1][r], hf);
+    for (int u = 0; u < 8; ++u) {
+      const int b = b0 + u * 32 + lane;
+      v[u] = b < nb ? __ldcg(p + (int64_t)b * stride) : 0.0;
     }
-    hpart[(int64_t)(2 * c) * G + blockIdx.x] = hv;
-    hpart[(int64_t)(2 * c + 1) * G + blockIdx.x] = hf;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (b0 + u * 32 < nb) s += v[u];   // uniform
+  }
+  return warp_sum(s);
+}
+
+// Sums over the block's rows of the values val[q][row], q < nv, into row[q]: one warp per value.
+template <int RB>
+SEED_DEV void row_sums(const double (*val)[RB], int nv, double *row) {
+  const int lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q < nv; q += RT / 32) {
+    double x = lane < RB ? val[q][lane] : 0.0;
+    if (RB > 32) x += val[q][(RB > 32 ? 32 : 0) + lane];
+    const double t = warp_sum(x);
+    if (lane == 0) row[q] = t;
   }
 }
 
-// H[q] = sum over blocks (block order) of hpart[q G + b], for this block's slice of q < 2k
-SEED_DEV void slice_reduce(const double *hpart, int k, double *H) {
-  const int G = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// After the barrier: this block's slice of H (values q < 2k of hpart summed over
+// the blocks) and, in every block, S[q] = the sum over blocks of region[b * kRunRegion + q], q <
+// nv; one warp per value, in block order.  Ends with a CTA barrier.
+SEED_DEV void gather(const double *hpart, int k, double *H, const double *region, int nv, double *S) {
+  const int G = gridDim.x, lane = threadIdx.x & 31;
   const int q0 = (int)((int64_t)2 * k * blockIdx.x / G), q1 = (int)((int64_t)2 * k * (blockIdx.x + 1) / G);
-  for (int q = q0 + warp; q < q1; q += PT / 32) {
-    const double t = warp_sum_partials(hpart + (int64_t)q * G, G, 1, 0);
-    if (lane == 0) H[q] = t;
+  for (int t = threadIdx.x >> 5; t < q1 - q0 + nv; t += RT / 32) {
+    const bool scalar = t < nv;
+    const int q = scalar ? t : q0 + t - nv;
+    const double x = scalar ? warp_sum_few(region + q, G, kRunRegion) : warp_sum_few(hpart + (int64_t)q * G, G, 1);
+    if (lane == 0) (scalar ? S : H)[q] = x;
+  }
+  __syncthreads();
+}
+
+// x 2^p as a 64-bit integer in two limbs hi 2^28 + lo, both with x's sign; x not finite or
+// zero: 0.  |x| 2^p < 2^57.  (p <= 1200: a subnormal x is cut off to zero.)
+SEED_DEV int2 limbs(double x, int p) {
+  const unsigned hw = (unsigned)__double2hiint(x);
+  const int be = (int)((hw >> 20) & 0x7ffu), sh = 1075 - be - p;   // mantissa (53 bits) >> sh
+  if (be == 0 || be == 2047 || sh > 53) return make_int2(0, 0);
+  const unsigned long long m =
+      (unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x);
+  const unsigned long long y = sh > 0 ? m >> sh : m << -sh;
+  const int s = (int)hw >> 31, hi = (int)(y >> 28), lo = (int)(y & 0xfffffffu);
+  return make_int2((hi ^ s) - s, (lo ^ s) - s);
+}
+// |x| < 2^(the result); a large negative number for zero
+SEED_DEV int exp2_above(double x) {
+  const int be = (__double2hiint(x) >> 20) & 0x7ff;
+  return be == 0 ? -1100 : be - 1022;
+}
+// (hi 2^56 + mid 2^28) 2^-p as a double
+SEED_DEV double limb_sum(long long hi, long long mid, int p) {
+  return scalbn((double)(hi + (mid >> 28)), 56 - p);
+}
+
+// hpart[(2 c + v) G + b] = sum over the block's rows r of V[c][row0 + r] y_v[r], c < k.  s_yl: the
+// limbs of y 2^(kYBits - ye[v]).  Up to four threads share a column's rows while k leaves
+// threads idle.
+template <int RB>
+SEED_DEV void col_dots(const int2 *sV, int kcap, const double *V, int64_t ldv, int64_t row0, int rows, int k,
+                       const double (*y)[RB], const int4 *s_yl, const int *ye, double *hpart) {
+  const int G = gridDim.x;
+  const int kf = k < kcap ? k : kcap;
+  const int lg = kf <= RT / 4 ? 2 : kf <= RT / 2 ? 1 : 0, part = threadIdx.x & ((1 << lg) - 1), nr = RB >> lg;
+  for (int c0 = 0; c0 < kf; c0 += RT >> lg) {   // uniform: the shuffles see whole warps
+    const int c = c0 + (threadIdx.x >> lg);
+    long long a0 = 0, m0 = 0, a1 = 0, m1 = 0;
+    if (c < kf) {
+      const int2 *vc = sV + (int64_t)c * (RB + 1) + part * nr;
+      const int4 *yl = s_yl + part * nr;
+#pragma unroll 4
+      for (int r = 0; r < nr; ++r) {   // rows past the end hold zeros
+        const int2 x = vc[r];
+        const int4 q = yl[r];
+        a0 = (long long)x.x * q.x + a0;
+        m0 = (long long)x.x * q.y + m0;
+        m0 = (long long)x.y * q.x + m0;
+        a1 = (long long)x.x * q.z + a1;
+        m1 = (long long)x.x * q.w + m1;
+        m1 = (long long)x.y * q.z + m1;
+      }
+    }
+    for (int o = 1; o < 1 << lg; o <<= 1) {
+      a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      m0 += __shfl_xor_sync(0xffffffffu, m0, o);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+      m1 += __shfl_xor_sync(0xffffffffu, m1, o);
+    }
+    if (c < kf && part == 0) {
+      hpart[(int64_t)(2 * c) * G + blockIdx.x] = limb_sum(a0, m0, kVBits + kYBits - ye[0]);
+      hpart[(int64_t)(2 * c + 1) * G + blockIdx.x] = limb_sum(a1, m1, kVBits + kYBits - ye[1]);
+    }
+  }
+  for (int c = kcap + threadIdx.x; c < k; c += RT) {
+    const double *vc = V + (int64_t)c * ldv + row0;
+    double h0 = 0.0, h1 = 0.0;
+    for (int r = 0; r < rows; ++r) {
+      const double x = vc[r];
+      h0 = fma(x, y[0][r], h0);
+      h1 = fma(x, y[1][r], h1);
+    }
+    hpart[(int64_t)(2 * c) * G + blockIdx.x] = h0;
+    hpart[(int64_t)(2 * c + 1) * G + blockIdx.x] = h1;
   }
 }
 
 // sub[v][r] = sum over c < k of V[c][row0 + r] H[2 c + v]: thread (r, g) of the
-// block (r = t mod RB, g = t / RB) sums the columns c = g, g + G, ... (G = PT /
-// RB groups) of row r, then each output adds its G group sums in group order --
-// G - 1 FP64 adds per output instead of a 31-add warp reduce-scatter per lane
-// (FP64 adds run at 2 per clock per SM on this part).
+// block (r = t mod RB, g = t / RB) sums the columns c = g, g + groups, ... of row r, then
+// each output adds its group sums in group order.  H comes from L2 once: as limbs with
+// one exponent per v into s_hl.
 template <int RB>
-SEED_DEV void rows_times_h(const double *V, int64_t ldv, int64_t row0, int rows, int k, const double *H,
-                           double (*sub)[RB], double (*sred)[2 * RB]) {
-  constexpr int kGroups = PT / RB;
-  const int r = threadIdx.x % RB, grp = threadIdx.x / RB;
-  double pv = 0.0, pf = 0.0;
-  if (r < rows) {
-    const double *vr = V + row0 + r;
-#pragma unroll 4
-    for (int c = grp; c < k; c += kGroups) {
-      const double x = vr[(int64_t)c * ldv];
-      pv = fma(x, __ldcg(H + 2 * c), pv);
-      pf = fma(x, __ldcg(H + 2 * c + 1), pf);
-    }
+SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V, int64_t ldv, int64_t row0, int rows,
+                           int k, const double *H, double (*sub)[RB], long long (*sred)[2 * RB], double (*stail)[2 * RB],
+                           int (*s_he)[2]) {
+  constexpr int kGroups = RT / RB;
+  const int kf = k < kcap ? k : kcap;   // columns in shared memory
+  int e0 = -1100, e1 = -1100;
+  for (int c = threadIdx.x; c < kf; c += RT) {
+    const double2 h = __ldcg(reinterpret_cast<const double2 *>(H) + c);
+    e0 = max(e0, exp2_above(h.x));
+    e1 = max(e1, exp2_above(h.y));
   }
-  sred[grp][r] = pv;
-  sred[grp][RB + r] = pf;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, o));
+    e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    s_he[threadIdx.x >> 5][0] = e0;
+    s_he[threadIdx.x >> 5][1] = e1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < RT / 32; ++w) {
+    e0 = max(e0, s_he[w][0]);
+    e1 = max(e1, s_he[w][1]);
+  }
+  for (int c = threadIdx.x; c < kf; c += RT) {
+    const double2 h = __ldcg(reinterpret_cast<const double2 *>(H) + c);
+    const int2 p = limbs(h.x, kHBits - e0), q = limbs(h.y, kHBits - e1);
+    s_hl[c] = make_int4(p.x, p.y, q.x, q.y);
+  }
+  __syncthreads();
+  const int r = threadIdx.x % RB, grp = threadIdx.x / RB;
+  long long a0 = 0, m0 = 0, a1 = 0, m1 = 0;
+#pragma unroll 4
+  for (int c = grp; c < kf; c += kGroups) {
+    const int2 x = sV[(int64_t)c * (RB + 1) + r];
+    const int4 q = s_hl[c];
+    a0 = (long long)x.x * q.x + a0;
+    m0 = (long long)x.x * q.y + m0;
+    m0 = (long long)x.y * q.x + m0;
+    a1 = (long long)x.x * q.z + a1;
+    m1 = (long long)x.x * q.w + m1;
+    m1 = (long long)x.y * q.z + m1;
+  }
+  // |V H| sums are below 2^(kVBits + kHBits) sqrt(k) in all: the shifted sums add up exactly
+  sred[grp][r] = a0 + (m0 >> 28);
+  sred[grp][RB + r] = a1 + (m1 >> 28);
+  const bool tail = k > kf;
+  if (tail) {
+    double pv = 0.0, pf = 0.0;
+    if (r < rows) {
+      const double *vr = V + row0 + r;
+      for (int c = kf + grp; c < k; c += kGroups) {
+        const double x = vr[(int64_t)c * ldv];
+        pv = fma(x, __ldcg(H + 2 * c), pv);
+        pf = fma(x, __ldcg(H + 2 * c + 1), pf);
+      }
+    }
+    stail[grp][r] = pv;
+    stail[grp][RB + r] = pf;
+  }
   __syncthreads();
   if ((int)threadIdx.x < 2 * RB) {
     const int q = threadIdx.x;
-    double t = sred[0][q];
+    long long t = sred[0][q];
 #pragma unroll
     for (int g2 = 1; g2 < kGroups; ++g2) t += sred[g2][q];
-    sub[q / RB][q % RB] = t;
+    double d = limb_sum(t, 0, kVBits + kHBits - (q < RB ? e0 : e1));
+    if (tail)
+      for (int g2 = 0; g2 < kGroups; ++g2) d += stail[g2][q];
+    sub[q / RB][q % RB] = d;
   }
   __syncthreads();
 }
 
 template <int RB>
-__global__ void __launch_bounds__(PT) k_seed_run_csr_reorth(SeedBufs<double> b, CsrOp op, double *f2, GridSync g,
+__global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, CsrOp op, double *f2, GridSync g,
                                                             double *bpart, double *hpart, double *H, int freq,
-                                                            int passes, int i_stop) {
-  static_assert(2 * RB % 32 == 0 && 2 * RB <= PT, "rows per block");
-  __shared__ double s_w[PT / 32][kRunRegion];
+                                                            int passes, int i_stop, int kcap) {
+  static_assert(2 * RB <= RT && RT % RB == 0, "rows per block");
+  __shared__ double s_val[kRunMaxRhs][RB];
   __shared__ double s_sum[kRunRegion];
   __shared__ double2 s_g[kRunMaxRhs];
   __shared__ double2 s_eta[kRunMaxRhs];
   __shared__ double s_y[2][RB];
+  __shared__ int4 s_yl[RB];
+  __shared__ int s_ye[2], s_he[RT / 32][2];
   __shared__ double s_sub[2][RB];
-  __shared__ double s_red[PT / RB][2 * RB];
+  __shared__ long long s_red[RT / RB][2 * RB];
+  __shared__ double s_tail[RT / RB][2 * RB];
   __shared__ LocalSeed L;
+  extern __shared__ int4 s_run[];
+  int4 *const s_hl = s_run;                                  // [kcap] limbs of H
+  int2 *const sV = reinterpret_cast<int2 *>(s_run + kcap);   // [kcap][RB + 1] limbs of this block's rows of V
   unsigned epoch = 0;
   int par = 0, reg = 0;
   local_load(b, L);
   const int nr = b.nrhs;   // <= kRunMaxRhs (checked by the host)
-  for (int j = threadIdx.x; j < nr; j += PT) s_eta[j] = b.eta[j];
+  for (int j = threadIdx.x; j < nr; j += RT) s_eta[j] = b.eta[j];
   __syncthreads();
   SeedBufs<double> bl = local_bufs(b, L);
   bl.eta = s_eta;
@@ -1426,139 +1584,213 @@ __global__ void __launch_bounds__(PT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     reg ^= 1;
     return r;
   };
+  // s_y and its limbs, from this thread's (v, f); ends with a CTA barrier
+  auto stage_y = [&](double yv, double yf) {
+    if ((int)threadIdx.x < RB) {
+      s_y[0][threadIdx.x] = own ? yv : 0.0;
+      s_y[1][threadIdx.x] = own ? yf : 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      int e0 = -1100, e1 = -1100;
+      for (int r = threadIdx.x; r < RB; r += 32) {
+        e0 = max(e0, exp2_above(s_y[0][r]));
+        e1 = max(e1, exp2_above(s_y[1][r]));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, o));
+        e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
+      }
+      for (int r = threadIdx.x; r < RB; r += 32) {
+        const int2 p = limbs(s_y[0][r], kYBits - e0), q = limbs(s_y[1][r], kYBits - e1);
+        s_yl[r] = make_int4(p.x, p.y, q.x, q.y);
+      }
+      if (threadIdx.x == 0) {
+        s_ye[0] = e0;
+        s_ye[1] = e1;
+      }
+    }
+    __syncthreads();
+  };
+  // column c of this block's rows of V in shared memory
+  auto keep = [&](int c, double v) {
+    if (c < kcap && (int)threadIdx.x < RB) sV[(int64_t)c * (RB + 1) + threadIdx.x] = limbs(own ? v : 0.0, kVBits);
+  };
+  const bool scalar = threadIdx.x == RT - 32;   // runs the recurrence's scalar code beside the others
+  double f = own ? b.f[e] : 0.0;   // this row's f, final
+  double hc = 0.0;                 // f in global memory is still to have hc v_{i-1} subtracted
+  double vlast = 0.0;              // this row's v_{i-1}
+  int il = L.st.i - 1;             // last finished step
+  for (int c = 0; c < il; ++c) keep(c, own ? b.V[(int64_t)c * ldv + e] : 0.0);   // (a run that starts later)
+  if (il > 0 && own) vlast = b.V[(int64_t)(il - 1) * ldv + e];
+  // The LU update's vectors of a step (w_i, x^1 += zeta_i w_i, x^j += eta^j w_i) wait for the next
+  // barrier's window: pend, with the step's v_i as it was before its reorthogonalization.
+  bool pend = false;
+  double pv = 0.0, pbp = 0.0;
+  auto update_wx = [&]() {
+    if (!pend) return;
+    pend = false;
+    if (!own) return;
+    const double zeta = L.st.zeta, inv_d = L.st.inv_delta;
+    const double we = il > 1 ? inv_d * fma(-pbp, b.w[e], pv) : inv_d * pv;
+    b.w[e] = we;
+    X[e] = fma(zeta, we, X[e]);
+    for (int j = 1; j < nr; ++j) X[e + j * ldx] = fma(s_eta[j].x, we, X[e + j * ldx]);
+  };
   for (;;) {
-    const int i = L.st.i;
-    if (!L.st.active || i >= i_stop) break;
-    const double inv_b = L.st.inv_beta;
-    const double bp = (i > 1) ? L.st.beta_prev : 0.0;
+    // ---- (A f)_e of the step that may follow, while the scalar thread ends the last one ----
     const double *fc = par ? f2 : b.f;
     double *fn = par ? b.f : f2;
-    double *vi = b.V + (int64_t)(i - 1) * ldv;
-    const double *vm = b.V + (int64_t)(i > 1 ? i - 2 : 0) * ldv;
-    // ---- v_i = f / beta_{i-1}; f = A v_i - beta_{i-1} v_{i-1}; alpha_i and g^j ----
-    double acc[kRunMaxRhs];
-#pragma unroll
-    for (int q = 0; q < kRunMaxRhs; ++q) acc[q] = 0.0;
-    double v = 0.0, fe = 0.0;
+    double sum = 0.0;
     if (own) {
-      double sum = 0.0;
+      const double *vm = b.V + (int64_t)(il > 0 ? il - 1 : 0) * ldv;
       if (cached) {
         double xv[kRowCache];
 #pragma unroll
         for (int q = 0; q < kRowCache; ++q) xv[q] = q < k1 - k0 ? __ldcg(fc + rc_col[q]) : 0.0;
+        if (hc != 0.0) {
+          double xm[kRowCache];
+#pragma unroll
+          for (int q = 0; q < kRowCache; ++q) xm[q] = q < k1 - k0 ? __ldcg(vm + rc_col[q]) : 0.0;
+#pragma unroll
+          for (int q = 0; q < kRowCache; ++q)
+            if (q < k1 - k0) xv[q] = fma(-hc, xm[q], xv[q]);
+        }
 #pragma unroll
         for (int q = 0; q < kRowCache; ++q)
           if (q < k1 - k0) sum = fma(rc_val[q], xv[q], sum);
       } else {
-        for (int32_t q = k0; q < k1; ++q) sum = fma(__ldg(op.vals + q), __ldcg(fc + __ldg(op.col_idx + q)), sum);
+        for (int32_t q = k0; q < k1; ++q) {
+          const int32_t c = __ldg(op.col_idx + q);
+          double x = __ldcg(fc + c);
+          if (hc != 0.0) x = fma(-hc, __ldcg(vm + c), x);
+          sum = fma(__ldg(op.vals + q), x, sum);
+        }
       }
-      v = inv_b * __ldcg(fc + e);
-      vi[e] = v;
-      double u = inv_b * sum;
-      if (i > 1) u = fma(-bp, vm[e], u);
-      fe = u;
-      acc[0] = v * u;
-#pragma unroll
-      for (int q = 1; q < kRunMaxRhs; ++q)
-        if (q < nr) acc[q] = v * b.R0[(int64_t)(q - 1) * b.ldr + e];
     }
-    {
-      double *r = region();
-      block_row<kRunMaxRhs>(acc, nr, r + (int64_t)blockIdx.x * kRunRegion, s_w);
-      if (!grid_sync(g, epoch)) return;
-      reduce_region(r, nr, s_sum);
+    __syncthreads();   // the scalar thread's part is done
+    const int i = L.st.i;
+    if (!L.st.active || i >= i_stop) break;
+    const double inv_b = L.st.inv_beta;
+    const double bp = (i > 1) ? L.st.beta_prev : 0.0;
+    double *vi = b.V + (int64_t)(i - 1) * ldv;
+    const bool ro = freq > 0 && i >= 2 && i % freq == 0;
+    const int k = i - 1;
+    // ---- v_i = f / beta_{i-1}; u = A v_i - beta_{i-1} v_{i-1}; alpha_i and g^j ----
+    double v = 0.0, u = 0.0;
+    if (own) {
+      v = inv_b * f;
+      u = inv_b * sum;
+      if (i > 1) u = fma(-bp, vlast, u);
+      vi[e] = v;   // (a reorthogonalizing step stores the final v_i over it)
     }
-    if (threadIdx.x == 0) {
+    if ((int)threadIdx.x < RB) {
+      s_val[0][threadIdx.x] = own ? v * u : 0.0;
+      for (int q = 1; q < nr; ++q) s_val[q][threadIdx.x] = own ? v * b.R0[(int64_t)(q - 1) * b.ldr + e] : 0.0;
+    }
+    double *r = region();
+    if (ro) {
+      stage_y(v, u);
+      col_dots<RB>(sV, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
+    } else {
+      __syncthreads();
+    }
+    row_sums<RB>(s_val, nr, r + (int64_t)blockIdx.x * kRunRegion);
+    grid_arrive(g, epoch);
+    update_wx();   // of step i - 1
+    if (!grid_wait(g, epoch)) return;
+    gather(hpart, ro ? k : 0, H, r, nr, s_sum);
+    // ---- f = u - alpha_i v_i; the LU update's scalars beside the next barrier ----
+    const double a = s_sum[0];
+    f = fma(-a, v, u);
+    pv = v;
+    pbp = bp;
+    il = i;
+    r = region();
+    if (!ro) {
+      keep(k, v);
+      if (own) fn[e] = f;
+      if ((int)threadIdx.x < RB) s_val[0][threadIdx.x] = own ? f * f : 0.0;
+      __syncthreads();
+      row_sums<RB>(s_val, 1, r + (int64_t)blockIdx.x * kRunRegion);
+    }
+    grid_arrive(g, epoch);
+    if (scalar) {
       for (int j = 1; j < nr; ++j) s_g[j] = c2(s_sum[j], 0.0);
       seed_step_scalars<double, false>(bl, i, s_sum[0], s_g);
     }
-    __syncthreads();
+    if (!grid_wait(g, epoch)) return;
     if (!L.st.active) break;   // delta_i <= 0
-    // ---- f -= alpha_i v_i; w_i; x^1 += zeta_i w_i; x^j += eta^j w_i ----
-    const bool ro = freq > 0 && i >= 2 && i % freq == 0;
-    {
-      const double a = L.st.alpha, zeta = L.st.zeta, inv_d = L.st.inv_delta;
-      double nf = 0.0;
-      if (own) {
-        fe = fma(-a, v, fe);
-        const double we = (i > 1) ? inv_d * fma(-bp, b.w[e], v) : inv_d * v;
-        b.w[e] = we;
-        X[e] = fma(zeta, we, X[e]);
-        for (int j = 1; j < nr; ++j) X[e + j * ldx] = fma(s_eta[j].x, we, X[e + j * ldx]);
-        nf = fe * fe;
-        if (!ro) fn[e] = fe;
-      }
-      if (!ro) {
-        double vv[1] = {nf};
-        double *r = region();
-        block_row<1>(vv, 1, r + (int64_t)blockIdx.x * kRunRegion, s_w);
-        if (!grid_sync(g, epoch)) return;
-        reduce_region(r, 1, s_sum);
-        if (threadIdx.x == 0) seed_finish<double, false>(bl, s_sum[0]);
-        __syncthreads();
-        par ^= 1;
-        continue;
-      }
+    pend = true;
+    if (!ro) {
+      gather(nullptr, 0, nullptr, r, 1, s_sum);
+      if (scalar) seed_finish<double, false>(bl, s_sum[0]);
+      hc = 0.0;
+      vlast = v;
+      par ^= 1;
+      continue;
     }
     // ---- reorthogonalization of v_i and f against V_{<i} (classical Gram-Schmidt, `passes` times) ----
-    const int k = i - 1;
-    if ((int)threadIdx.x < RB) {
-      s_y[0][threadIdx.x] = own ? v : 0.0;
-      s_y[1][threadIdx.x] = own ? fe : 0.0;
-    }
-    __syncthreads();
-    col_dots<RB>(b.V, ldv, row0, rows, k, s_y, hpart);
-    for (int pass = 0; pass < passes; ++pass) {
-      if (!grid_sync(g, epoch)) return;
-      slice_reduce(hpart, k, H);
-      if (!grid_sync(g, epoch)) return;
-      rows_times_h<RB>(b.V, ldv, row0, rows, k, H, s_sub, s_red);
-      if ((int)threadIdx.x < RB) {
-        s_y[0][threadIdx.x] = fma(-1.0, s_sub[0][threadIdx.x], s_y[0][threadIdx.x]);
-        s_y[1][threadIdx.x] = fma(-1.0, s_sub[1][threadIdx.x], s_y[1][threadIdx.x]);
+    double inv = 0.0, svf = 0.0;   // 1 / ||v_i|| and v_i^H f of the normalization
+    for (int pass = 0;; ++pass) {
+      rows_times_h<RB>(sV, kcap, s_hl, b.V, ldv, row0, rows, k, H, s_sub, s_red, s_tail, s_he);
+      if (own) {
+        const double sv = s_sub[0][threadIdx.x], sf = s_sub[1][threadIdx.x];
+        v -= sv;
+        f -= pass == 0 ? fma(-a, sv, sf) : sf;   // pass 0: V V^H u - alpha_i V V^H v_i
       }
-      __syncthreads();
-      if (pass + 1 < passes) col_dots<RB>(b.V, ldv, row0, rows, k, s_y, hpart);
-    }
-    v = own ? s_y[0][threadIdx.x] : 0.0;
-    fe = own ? s_y[1][threadIdx.x] : 0.0;
-    // ---- v_i /= ||v_i||, then f -= (v_i^H f) v_i, `passes` times; ||f||^2 ends the step.
-    // ||v_i||^2 and v_i^H f come from one reduction (h = (v_i^H f) / ||v_i|| before
-    // the scaling: the first projection's coefficient, rounded in another order) ----
-    {
-      double vv[2] = {v * v, v * fe};
-      double *r = region();
-      block_row<2>(vv, 2, r + (int64_t)blockIdx.x * kRunRegion, s_w);
-      if (!grid_sync(g, epoch)) return;
-      reduce_region(r, 2, s_sum);
-    }
-    {
-      const double inv = 1.0 / sqrt(s_sum[0]);
-      v = inv * v;
-      fe = fma(-(s_sum[1] * inv), v, fe);
-    }
-    if (own) vi[e] = v;
-    for (int pass = 1; pass <= passes; ++pass) {
-      // pass < passes: h = v_i^H f, then f -= h v_i; pass == passes: ||f||^2 (f final: stored first)
-      if (pass == passes && own) fn[e] = fe;
-      double vv[1] = {pass < passes ? v * fe : fe * fe};
-      double *r = region();
-      block_row<1>(vv, 1, r + (int64_t)blockIdx.x * kRunRegion, s_w);
-      if (!grid_sync(g, epoch)) return;
-      reduce_region(r, 1, s_sum);
-      if (pass < passes) {
-        fe = fma(-s_sum[0], v, fe);
+      if (pass > 0) break;
+      if ((int)threadIdx.x < RB) {
+        s_val[0][threadIdx.x] = own ? v * v : 0.0;
+        s_val[1][threadIdx.x] = own ? v * f : 0.0;
+      }
+      if (passes > 1) {
+        stage_y(v, f);
+        col_dots<RB>(sV, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
       } else {
-        if (threadIdx.x == 0) seed_finish<double, false>(bl, s_sum[0]);
         __syncthreads();
       }
+      row_sums<RB>(s_val, 2, r + (int64_t)blockIdx.x * kRunRegion);
+      grid_arrive(g, epoch);
+      update_wx();   // of this step
+      if (!grid_wait(g, epoch)) return;
+      gather(hpart, passes > 1 ? k : 0, H, r, 2, s_sum);
+      svf = s_sum[1];
+      if (passes > 1) grid_arrive(g, epoch);
+      inv = 1.0 / sqrt(s_sum[0]);
+      if (passes == 1) break;
+      if (!grid_wait(g, epoch)) return;
     }
+    // ---- v_i /= ||v_i||, f -= (v_i^H f) v_i; two passes: again, with the coefficient
+    // and ||f||^2 from one sum (the readers of f subtract) ----
+    v = inv * v;
+    f = fma(-(svf * inv), v, f);
+    keep(k, v);
+    if (own) {
+      vi[e] = v;
+      fn[e] = f;
+    }
+    if ((int)threadIdx.x < RB) {
+      s_val[0][threadIdx.x] = own ? f * f : 0.0;
+      s_val[1][threadIdx.x] = own ? v * f : 0.0;
+    }
+    r = region();
+    __syncthreads();
+    row_sums<RB>(s_val, 2, r + (int64_t)blockIdx.x * kRunRegion);
+    if (!grid_sync(g, epoch)) return;
+    gather(nullptr, 0, nullptr, r, 2, s_sum);
+    hc = passes > 1 ? s_sum[1] : 0.0;
+    if (hc != 0.0) f = fma(-hc, v, f);
+    if (scalar) seed_finish<double, false>(bl, fmax(0.0, fma(-hc, hc, s_sum[0])));
+    vlast = v;
     par ^= 1;
   }
-  seed_leave<double>(b, L, par ? f2 : b.f, i_stop);
   __syncthreads();
+  update_wx();
+  if (L.st.active && L.st.i == i_stop && own) b.f[e] = f;   // the next step starts from f in b.f
   if (blockIdx.x == 0)
-    for (int j = threadIdx.x; j < nr; j += PT) b.eta[j] = s_eta[j];
+    for (int j = threadIdx.x; j < nr; j += RT) b.eta[j] = s_eta[j];
   local_store(b, L);
 }
 
@@ -2010,9 +2242,14 @@ __global__ void __launch_bounds__(PT) k_cg_run_csr_small(CsrOp op, const CallArg
   }
 }
 
+static const void *small_cg_kernel(int rb) {
+  return rb == 16 ? (const void *)k_cg_run_csr_small<16> : rb == 32 ? (const void *)k_cg_run_csr_small<32>
+                                                                    : (const void *)k_cg_run_csr_small<64>;
+}
+
 int small_cg_grid_cap(int sm_count, int rb) {
   int per_sm = 0;
-  const void *k = rb == 16 ? (const void *)k_cg_run_csr_small<16> : (const void *)k_cg_run_csr_small<32>;
+  const void *k = small_cg_kernel(rb);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, PT, 0) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -2027,8 +2264,7 @@ cudaError_t launch_cg_run_csr_small(const CsrOp &op, const CallArgs *call, doubl
   CsrOp o = op;
   CgCols cc = c;
   void *args[] = {&o, &call, &R, &P, &P2, &Q, &ld, &cc, &g, &bpart};
-  const void *k = rb == 16 ? (const void *)k_cg_run_csr_small<16> : (const void *)k_cg_run_csr_small<32>;
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(PT), args, 0, s);
+  return cudaLaunchCooperativeKernel(small_cg_kernel(rb), dim3(grid), dim3(PT), args, 0, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -2141,10 +2377,24 @@ cudaError_t launch_barrier_timeout_check(GridSync g, cudaStream_t s) {
   return cudaLaunchCooperativeKernel((const void *)k_barrier_timeout_check, dim3(2), dim3(PT), args, 0, s);
 }
 
+static const void *reorth_run_kernel(int rb) {
+  return rb == 16 ? (const void *)k_seed_run_csr_reorth<16> : rb == 32 ? (const void *)k_seed_run_csr_reorth<32>
+                                                                       : (const void *)k_seed_run_csr_reorth<64>;
+}
+// columns of V whose rows a block keeps in shared memory, and the bytes they take
+static int reorth_run_cols(int rb, int m) {
+  const int most = kRunSmem / ((rb + 1) * (int)sizeof(int2) + (int)sizeof(int4));
+  return m < most ? m : most;
+}
+static size_t reorth_run_smem(int rb, int kcap) {
+  return (size_t)kcap * ((rb + 1) * sizeof(int2) + sizeof(int4));
+}
+
 int reorth_run_grid_cap(int sm_count, int rb) {
   int per_sm = 0;
-  const void *k = rb == 16 ? (const void *)k_seed_run_csr_reorth<16> : (const void *)k_seed_run_csr_reorth<32>;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, PT, 0) != cudaSuccess) {
+  const void *k = reorth_run_kernel(rb);
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, RT, kRunSmem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -2157,9 +2407,9 @@ cudaError_t launch_seed_run_csr_reorth(const SeedBufs<double> &b, const CsrOp &o
                                        int rb, int grid, cudaStream_t s) {
   SeedBufs<double> bb = b;
   CsrOp o = op;
-  void *args[] = {&bb, &o, &f2, &g, &bpart, &hpart, &H, &freq, &passes, &i_stop};
-  const void *k = rb == 16 ? (const void *)k_seed_run_csr_reorth<16> : (const void *)k_seed_run_csr_reorth<32>;
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(PT), args, 0, s);
+  int kcap = reorth_run_cols(rb, i_stop);
+  void *args[] = {&bb, &o, &f2, &g, &bpart, &hpart, &H, &freq, &passes, &i_stop, &kcap};
+  return cudaLaunchCooperativeKernel(reorth_run_kernel(rb), dim3(grid), dim3(RT), args, reorth_run_smem(rb, kcap), s);
 }
 
 cudaError_t launch_cg_run_csr(const CsrOp &op, const CallArgs *call, double *R, double *P, double *Q, int64_t ld,

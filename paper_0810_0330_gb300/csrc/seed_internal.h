@@ -344,7 +344,7 @@ cudaError_t launch_seed_run_csr(const SeedBufs<double> &b, const CsrOp &op, doub
                                 int i_stop, int grid, cudaStream_t s);
 // Small real CSR problems reorthogonalizing every freq (1..7) steps, streaming
 // seeding, nrhs <= 16: the whole seed run in one launch of ceil(n / rb) blocks
-// (rb = 16 or 32 rows per block).  bpart: 2 x grid x 32 doubles; hpart:
+// (rb = 16, 32 or 64 rows per block).  bpart: 2 x grid x 32 doubles; hpart:
 // 2 x (m_max + 1) x grid doubles; H: 2 x (m_max + 1) doubles.
 constexpr int64_t kReorthRunMaxN = 32 * 304;
 constexpr int kReorthRunMaxRhs = 16;
