@@ -312,7 +312,8 @@ SEED_DEV bool seed_beta_step(const SeedBufs<T> &bl, const double *parts, int npa
 template <class T>
 SEED_DEV void seed_leave(const SeedBufs<T> &b, const LocalSeed &L, const T *f, int i_stop) {
   if (!L.st.active || L.st.i != i_stop || f == b.f) return;
-  for (int64_t e = (int64_t)blockIdx.x * PT + threadIdx.x; e < b.n; e += (int64_t)gridDim.x * PT) b.f[e] = __ldcg(f + e);
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < b.n; e += step) b.f[e] = __ldcg(f + e);
 }
 
 // FP64 Wilson run: five warps per block.  Warps 0-3 are the tile warps of the
@@ -1195,6 +1196,12 @@ __global__ void __launch_bounds__(kSiteThreads32 + 32, 1) k_seed_run_wilson32s(S
   local_store(b, L);
 }
 
+// Threads per block of the CSR seed run: with csr_seed_grid's blocks about four rows per
+// thread, whose loads follow one another.  48^3 grid, 139 steps: 4.41 ms with 128
+// threads, 3.42 with 256, 3.19 with 512; a batch of 12 problems side by side 26.7, 25.6 and 27.4
+// ms (512: their blocks no longer fit the GPU together).
+constexpr int CRT = 256;
+
 // Phase 3 of the CSR run: f -= alpha_i v_i, w_i (also into column i - blk0 of
 // Wb), x^1 and ||f||^2; one value per block, reduced in block order by every
 // block after the barrier, then the end of the step.
@@ -1206,7 +1213,7 @@ SEED_DEV bool seed_update_step(const SeedBufs<T> &b, const SeedBufs<T> &bl, T *f
   T *const X = reinterpret_cast<T *>(b.call->X);
   T *const wcol = b.Wb != nullptr ? b.Wb + (int64_t)(i - L.st.blk0) * b.ldv : nullptr;
   typename Sc<T>::A acc = 0;
-  for (int64_t e = (int64_t)blockIdx.x * PT + threadIdx.x; e < b.n; e += (int64_t)gridDim.x * PT) {
+  for (int64_t e = (int64_t)blockIdx.x * CRT + threadIdx.x; e < b.n; e += (int64_t)gridDim.x * CRT) {
     const T v = __ldcg(vi + e), f0 = __ldcg(f + e), x0 = __ldcg(X + e);
     const T wp = (i > 1) ? __ldcg(b.w + e) : Sc<T>::zero();
     const T fe = Sc<T>::axpy(-a, v, f0);
@@ -1218,7 +1225,7 @@ SEED_DEV bool seed_update_step(const SeedBufs<T> &b, const SeedBufs<T> &bl, T *f
     acc = Sc<T>::nrm2(fe, acc);
   }
   double vv[1] = {(double)acc};
-  block_sum<1, PT>(vv, s_red);
+  block_sum<1, CRT>(vv, s_red);
   if (threadIdx.x == 0) bpart[blockIdx.x] = vv[0];
   return seed_beta_step<T>(bl, bpart, gridDim.x, i, L, g, epoch);
 }
@@ -1229,9 +1236,9 @@ SEED_DEV bool seed_update_step(const SeedBufs<T> &b, const SeedBufs<T> &bl, T *f
 // for the mixed-precision path (FP32 matrix values and vectors; per-thread
 // sums in FP32, block and grid sums and every scalar in FP64).
 template <class T>
-__global__ void __launch_bounds__(PT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> op, T *f2, GridSync g, double *bpart,
+__global__ void __launch_bounds__(CRT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> op, T *f2, GridSync g, double *bpart,
                                                       int i_stop) {
-  __shared__ double s_red[PT / 32];
+  __shared__ double s_red[CRT / 32];
   __shared__ LocalSeed L;
   unsigned epoch = 0;
   int par = 0;
@@ -1247,7 +1254,7 @@ __global__ void __launch_bounds__(PT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> op
     T *vi = b.V + (int64_t)(i - 1) * b.ldv;
     const T *vm = b.V + (int64_t)(i > 1 ? i - 2 : 0) * b.ldv;
     T apart = 0;
-    for (int64_t r = (int64_t)blockIdx.x * PT + threadIdx.x; r < b.n; r += (int64_t)gridDim.x * PT) {
+    for (int64_t r = (int64_t)blockIdx.x * CRT + threadIdx.x; r < b.n; r += (int64_t)gridDim.x * CRT) {
       const int32_t k0 = __ldg(op.row_ptr + r), k1 = __ldg(op.row_ptr + r + 1);
       T sum = 0;
       for (int32_t k = k0; k < k1; ++k) sum = fma(__ldg(op.vals + k), fc[__ldg(op.col_idx + k)], sum);
@@ -1264,7 +1271,7 @@ __global__ void __launch_bounds__(PT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> op
     double *apartials = bpart + (int64_t)gridDim.x * 32;
     {
       double vv[1] = {(double)apart};
-      block_sum<1, PT>(vv, s_red);
+      block_sum<1, CRT>(vv, s_red);
       if (threadIdx.x == 0) apartials[blockIdx.x] = vv[0];   // by blockIdx: fixed order
     }
     if (!seed_alpha_step<T>(bl, apartials, gridDim.x, 1, false, i, L, g, epoch)) return;
@@ -2292,7 +2299,7 @@ int persistent_grid(int kind, int sm_count, bool cg, bool fp32) {
   else if (fp32) k = kind == 0 ? (const void *)k_seed_run_csr<float> : (const void *)k_seed_run_wilson32;
   else k = kind == 0 ? (const void *)k_seed_run_csr<double> : (const void *)k_seed_run_wilson;
   const bool wil = !cg && kind == 1;   // the Wilson seed runs: five warps, resident tiles
-  const int threads = wil ? PTW : PT;
+  const int threads = wil ? PTW : cg ? PT : CRT;
   if (wil && seed_run_wilson_smem_attr() != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -2332,14 +2339,14 @@ cudaError_t launch_seed_run_csr(const SeedBufs<double> &b, const CsrOp &op, doub
   SeedBufs<double> bb = b;
   CsrOp o = op;
   void *args[] = {&bb, &o, &f2, &g, &bpart, &i_stop};
-  return cudaLaunchCooperativeKernel((const void *)k_seed_run_csr<double>, dim3(grid), dim3(PT), args, 0, s);
+  return cudaLaunchCooperativeKernel((const void *)k_seed_run_csr<double>, dim3(grid), dim3(CRT), args, 0, s);
 }
 cudaError_t launch_seed_run_csr32(const SeedBufs<float> &b, const CsrOp32 &op, float *f2, GridSync g, double *bpart,
                                   int i_stop, int grid, cudaStream_t s) {
   SeedBufs<float> bb = b;
   CsrOp32 o = op;
   void *args[] = {&bb, &o, &f2, &g, &bpart, &i_stop};
-  return cudaLaunchCooperativeKernel((const void *)k_seed_run_csr<float>, dim3(grid), dim3(PT), args, 0, s);
+  return cudaLaunchCooperativeKernel((const void *)k_seed_run_csr<float>, dim3(grid), dim3(CRT), args, 0, s);
 }
 cudaError_t launch_seed_run_wilson32(const SeedBufs<float2> &b, const WilsonOp32 &op, float2 *tbuf, GridSync g,
                                      double *tpart, int i_stop, int grid, cudaStream_t s) {
