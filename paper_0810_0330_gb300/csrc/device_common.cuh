@@ -128,7 +128,8 @@ SEED_DEV double warp_sum(double x) {
   return x;
 }
 
-// Sum of K values over the block; the result is returned to every thread.
+// Sum of K values over the block, valid in the first warp (the other warps' copies
+// would cost as many FP64 adds again: 64 clocks of a sub-partition's FP64 unit each).
 // smem must hold K * (NT/32) doubles.
 template <int K, int NT>
 SEED_DEV void block_sum(double (&v)[K], double *smem) {
@@ -140,12 +141,14 @@ SEED_DEV void block_sum(double (&v)[K], double *smem) {
     if (lane == 0) smem[k * NW + warp] = x;
   }
   __syncthreads();
+  if (warp == 0) {
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double s = 0.0;
+    for (int k = 0; k < K; ++k) {
+      double s = smem[k * NW];
 #pragma unroll
-    for (int w = 0; w < NW; ++w) s += smem[k * NW + w];
-    v[k] = s;
+      for (int w = 1; w < NW; ++w) s += smem[k * NW + w];
+      v[k] = s;
+    }
   }
   __syncthreads();
 }
@@ -168,7 +171,8 @@ SEED_DEV bool last_block_done(unsigned *ticket, unsigned expected) {
 }
 
 // In the last block: sum partial[b*stride + k] over b = 0..nb-1 in a fixed
-// order; returned to every thread.  smem: NT/32 doubles.
+// order, valid in the first warp; adds whose operand is zero for want of partials are
+// left out (nb is uniform).  smem: NT/32 doubles.
 template <int NT>
 SEED_DEV double sum_partials(const double *partial, int nb, int stride, int k, double *smem) {
   double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -180,9 +184,14 @@ SEED_DEV double sum_partials(const double *partial, int nb, int stride, int k, d
       v[u] = b < nb ? __ldcg(partial + (int64_t)b * stride + k) : 0.0;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) s[u] += v[u];
+    for (int u = 0; u < 4; ++u) {
+      if (b0 == 0) s[u] = v[u];
+      else if (b0 + u * NT < nb) s[u] += v[u];
+    }
   }
-  double v[1] = {(s[0] + s[1]) + (s[2] + s[3])};
+  double v[1] = {s[0]};
+  if (nb > NT) v[0] = s[0] + s[1];
+  if (nb > 2 * NT) v[0] += s[2] + s[3];
   block_sum<1, NT>(v, smem);
   return v[0];
 }
@@ -221,9 +230,15 @@ SEED_DEV double warp_sum_partials(const double *partial, int nb, int stride, int
       v[u] = b < nb ? __ldcg(partial + (int64_t)b * stride + k) : 0.0;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) s[u] += v[u];
+    for (int u = 0; u < 8; ++u) {
+      if (b0 == 0) s[u] = v[u];
+      else if (b0 + u * 32 < nb) s[u] += v[u];   // uniform: no adds of absent partials
+    }
   }
-  const double t = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  double t = s[0];
+  if (nb > 32) t += s[1];
+  if (nb > 64) t += s[2] + s[3];
+  if (nb > 128) t += (s[4] + s[5]) + (s[6] + s[7]);
   return warp_sum(t);
 }
 

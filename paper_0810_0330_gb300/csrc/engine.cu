@@ -546,7 +546,7 @@ int run_length(const seed_params &p) {
   return best >= 8 ? best : 16;
 }
 
-// Blocks of a persistent CSR seed run: about 8 rows per thread, at least 16
+// Blocks of a persistent CSR seed run: about 1024 rows per block, at least 16
 // blocks, at most the occupancy-derived grid.  Small problems get small grids
 // (cheaper barriers, and in a batch several problems' runs fit side by side).
 int csr_seed_grid(const seed_ctx *ctx) {
@@ -822,17 +822,17 @@ int issue_cg_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, const 
     // p's blocks are in F: t = D p, q = D^H t with alpha, the residual, then x and p (with its blocks)
     int4 *Fb = ctx->F + (int64_t)c0 * ld, *Tb = fix_T(ctx) + (int64_t)c0 * ld;
     int32_t *Fe = ctx->Fe + (int64_t)c0 * (ld / 12), *Te = fix_Te(ctx) + (int64_t)c0 * (ld / 12);
-    const FixDot dot{P, ctx->dotpart + (int64_t)c0 * (ld / 192), tickets, c.rho, c.alpha};
+    const CgDot<double2> dot{P, ctx->dotpart + (int64_t)c0 * (ld / 192), tickets, c.rho, c.alpha};
     launch_dslash_fix(ctx->wfix, +1, Fb, Fe, ld, Tb, Te, nullptr, 0, c.nc, c.active, s);
     launch_dslash_fix(ctx->wfix, -1, Tb, Te, ld, nullptr, nullptr, Q, ld, c.nc, c.active, s, &dot);
-    launch_cg_residual(n, R, Q, ld, c, partials, tickets, s);
+    launch_cg_residual<T>(n, R, Q, ld, c, partials, tickets, s);
     launch_cg_xp_fix(ctx->wfix, call, R, P, ld, Fb, Fe, c, s);
     return 4;
   } else {
     launch_csr_spmv(ctx->csr, P, ld, Q, ld, c.nc, c.active, s);
     launch_cg_alpha<T>(n, P, Q, ld, c, partials, tickets, s);
-    launch_cg_update<T>(n, call, R, P, Q, ld, c, partials, tickets, s);
-    launch_cg_p<T>(n, R, P, ld, c, s);
+    launch_cg_residual<T>(n, R, Q, ld, c, partials, tickets, s);
+    launch_cg_xp<T>(n, call, R, P, ld, c, s);
     return 4;
   }
 }
@@ -842,7 +842,7 @@ CgCols cg_sub(const CgCols &c, int c0, int nc) {
   CgCols v = c;
   v.nc = nc;
   for (double **p : {&v.rho, &v.alpha, &v.beta, &v.bnorm, &v.relres, &v.rupd}) *p += c0;
-  for (int32_t **p : {&v.active, &v.iters, &v.reached, &v.restarts, &v.converged, &v.needs_check, &v.mvps, &v.upd})
+  for (int32_t **p : {&v.active, &v.iters, &v.reached, &v.restarts, &v.converged, &v.needs_check, &v.mvps, &v.upd, &v.stepped})
     *p += c0;
   return v;
 }
@@ -911,6 +911,7 @@ CgCols cg_cols(seed_ctx *ctx, int nc) {
   c.needs_check = q + 5 * kMaxRhs;
   c.mvps = q + 6 * kMaxRhs;
   c.upd = q + 7 * kMaxRhs;
+  c.stepped = q + 8 * kMaxRhs;
   c.tol = ctx->prm.tol_rest;
   c.tol_check = 1.5 * ctx->prm.tol_rest;
   c.maxit = ctx->prm.maxit_rest;
@@ -1375,20 +1376,18 @@ int issue_mixed_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, con
   const int64_t n = ctx->nv, ld = ctx->ldv;
   T32 *P = (T32 *)ctx->P32 + (int64_t)c0 * ld, *Q = (T32 *)ctx->Q32 + (int64_t)c0 * ld;
   T32 *R = (T32 *)ctx->R32 + (int64_t)c0 * ld;
-  int k;
-  if (ctx->kind == 0) {
-    launch_csr_spmv32(ctx->csr32, (const float *)P, ld, (float *)Q, ld, c.nc, c.active, s);
-    k = 1;
+  if constexpr (std::is_same_v<T32, float>) {
+    launch_csr_spmv32(ctx->csr32, P, ld, Q, ld, c.nc, c.active, s);
+    launch_cg_alpha<T32>(n, P, Q, ld, c, partials, tickets, s);
   } else {
     float2 *Tb = (float2 *)ctx->T32 + (int64_t)c0 * ld;
-    launch_wilson_dslash32(ctx->wil32, +1, (const float2 *)P, ld, Tb, ld, c.nc, c.active, true, s);
-    launch_wilson_dslash32(ctx->wil32, -1, Tb, ld, (float2 *)Q, ld, c.nc, c.active, true, s);
-    k = 2;
+    const CgDot<float2> dot{P, ctx->dotpart + (int64_t)c0 * (ld / 192), tickets, c.rho, c.alpha};
+    launch_wilson_dslash32(ctx->wil32, +1, P, ld, Tb, ld, c.nc, c.active, true, s);
+    launch_wilson_dslash32(ctx->wil32, -1, Tb, ld, Q, ld, c.nc, c.active, true, s, &dot);
   }
-  launch_cg_alpha<T32>(n, P, Q, ld, c, partials, tickets, s);
-  launch_cg_update<T32>(n, call, R, P, Q, ld, c, partials, tickets, s);
-  launch_cg_p<T32>(n, R, P, ld, c, s);
-  return k + 3;
+  launch_cg_residual<T32>(n, R, Q, ld, c, partials, tickets, s);
+  launch_cg_xp<T32>(n, call, R, P, ld, c, s);
+  return 4;
 }
 
 // CG on columns c0..c0+nc-1 of B and X (FP64) to ||b - A x|| <= tol ||b||

@@ -853,8 +853,9 @@ __global__ void __launch_bounds__(NT) k_cg_alpha(int64_t n, const T *P, const T 
   double *part = partials + (int64_t)col * gridDim.x;
   if (threadIdx.x == 0) part[blockIdx.x] = v[0];
   if (!last_block_done(tickets + kColTicket + col, gridDim.x)) return;
+  const double rho = __ldcg(c.rho + col);
   const double pq = sum_partials<NT>(part, gridDim.x, 1, 0, sm);
-  if (threadIdx.x == 0) c.alpha[col] = c.rho[col] / pq;
+  if (threadIdx.x == 0) c.alpha[col] = rho / pq;
 }
 
 // x += alpha p; r -= alpha q; test ||r|| <= tol ||b||; beta = rho'/rho
@@ -882,39 +883,62 @@ __global__ void __launch_bounds__(NT) k_cg_update(int64_t n, const CallArgs *cal
   double *part = partials + (int64_t)col * gridDim.x;
   if (threadIdx.x == 0) part[blockIdx.x] = v[0];
   if (!last_block_done(tickets + kColTicket + col, gridDim.x)) return;
+  const CgState t = cg_state(c, col);
   const double rr = sum_partials<NT>(part, gridDim.x, 1, 0, sm);
-  if (threadIdx.x == 0) cg_update_tail(c, col, rr);
+  cg_update_tail(c, col, rr, t);
 }
 
-// The same without x, which launch_cg_xp_fix (wilson_fixed.cu) updates with p;
-// upd[col] tells it which columns did an iteration.
-__global__ void __launch_bounds__(NT) k_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, CgCols c,
+// The same without x, which the kernel that updates p does with p at hand (one read of p
+// less); stepped[col] tells it which columns did an iteration.
+template <class T>
+__global__ void __launch_bounds__(NT) k_cg_residual(int64_t n, T *R, const T *Q, int64_t ld, CgCols c,
                                                     double *partials, unsigned *tickets) {
   __shared__ double sm[NT / 32];
   const int col = blockIdx.y;
   if (!c.active[col]) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) c.upd[col] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) c.stepped[col] = 0;
     return;
   }
   R += (int64_t)col * ld;
   Q += (int64_t)col * ld;
   const double a = c.alpha[col];
-  double acc = 0.0;
+  typename Sc<T>::A acc = 0;
 #pragma unroll 4
   GRID_STRIDE(e, n) {
-    const double2 r = Sc<double2>::axpy(-a, Q[e], R[e]);
+    const T r = Sc<T>::axpy(-a, Q[e], R[e]);
     R[e] = r;
-    acc = Sc<double2>::nrm2(r, acc);
+    acc = Sc<T>::nrm2(r, acc);
   }
-  double v[1] = {acc};
+  double v[1] = {(double)acc};
   block_sum<1, NT>(v, sm);
   double *part = partials + (int64_t)col * gridDim.x;
   if (threadIdx.x == 0) part[blockIdx.x] = v[0];
   if (!last_block_done(tickets + kColTicket + col, gridDim.x)) return;
+  const CgState t = cg_state(c, col);
   const double rr = sum_partials<NT>(part, gridDim.x, 1, 0, sm);
-  if (threadIdx.x == 0) {
-    c.upd[col] = 1;
-    cg_update_tail(c, col, rr);
+  if (threadIdx.x == 0) c.stepped[col] = 1;
+  cg_update_tail(c, col, rr, t);
+}
+
+// x += alpha p of the columns that did an iteration; p = r + beta p of those still active
+template <class T>
+__global__ void __launch_bounds__(NT) k_cg_xp(int64_t n, const CallArgs *call, const T *R, T *P, int64_t ld, CgCols c) {
+  const int col = blockIdx.y;
+  if (!c.stepped[col]) return;
+  T *X = reinterpret_cast<T *>(call->X) + (int64_t)(col + call->col0) * call->ldx;
+  R += (int64_t)col * ld;
+  P += (int64_t)col * ld;
+  const double a = c.alpha[col];
+  if (c.active[col]) {
+    const double be = c.beta[col];
+#pragma unroll 4
+    GRID_STRIDE(e, n) {
+      const T p = P[e];
+      X[e] = Sc<T>::axpy(a, p, X[e]);
+      P[e] = Sc<T>::axpy(be, p, R[e]);
+    }
+  } else {
+    GRID_STRIDE(e, n) X[e] = Sc<T>::axpy(a, P[e], X[e]);
   }
 }
 
@@ -992,10 +1016,16 @@ void launch_cg_update(int64_t n, const CallArgs *call, T *R, const T *P, const T
   dim3 g((unsigned)col_blocks(n, c.nc), (unsigned)c.nc);
   k_cg_update<T><<<g, NT, 0, s>>>(n, call, R, P, Q, ld, c, partials, tickets);
 }
-void launch_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, const CgCols &c, double *partials,
-                        unsigned *tickets, cudaStream_t s) {
+template <class T>
+void launch_cg_residual(int64_t n, T *R, const T *Q, int64_t ld, const CgCols &c, double *partials, unsigned *tickets,
+                        cudaStream_t s) {
   dim3 g((unsigned)col_blocks(n, c.nc), (unsigned)c.nc);
-  k_cg_residual<<<g, NT, 0, s>>>(n, R, Q, ld, c, partials, tickets);
+  k_cg_residual<T><<<g, NT, 0, s>>>(n, R, Q, ld, c, partials, tickets);
+}
+template <class T>
+void launch_cg_xp(int64_t n, const CallArgs *call, const T *R, T *P, int64_t ld, const CgCols &c, cudaStream_t s) {
+  dim3 g((unsigned)col_blocks(n, c.nc), (unsigned)c.nc);
+  k_cg_xp<T><<<g, NT, 0, s>>>(n, call, R, P, ld, c);
 }
 template <class T>
 void launch_cg_p(int64_t n, const T *R, T *P, int64_t ld, const CgCols &c, cudaStream_t s) {
@@ -1030,6 +1060,10 @@ void launch_cg_check(int64_t n, const T *B, int64_t ldb, const T *Q, int64_t ldq
   template void launch_cg_update<T>(int64_t, const CallArgs *, T *, const T *, const T *, int64_t, const CgCols &, \
                                     double *, unsigned *, cudaStream_t);                                         \
   template void launch_cg_p<T>(int64_t, const T *, T *, int64_t, const CgCols &, cudaStream_t);                  \
+  template void launch_cg_residual<T>(int64_t, T *, const T *, int64_t, const CgCols &, double *, unsigned *,    \
+                                      cudaStream_t);                                                             \
+  template void launch_cg_xp<T>(int64_t, const CallArgs *, const T *, T *, int64_t, const CgCols &,              \
+                                cudaStream_t);                                                                   \
   template void launch_cg_check<T>(int64_t, const T *, int64_t, const T *, int64_t, T *, int64_t,                \
                                    const CgCols &, double *, unsigned *, cudaStream_t);
 

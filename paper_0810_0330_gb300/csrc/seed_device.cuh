@@ -102,26 +102,40 @@ SEED_DEV void seed_finish(const SeedBufs<T> &b, double sumsq) {
   }
 }
 
-// Lockstep CG, after x += alpha p, r -= alpha q and rr = ||r||^2 (thread 0 of
-// the block that reduced column col): count the iteration, stop the column
-// when ||r|| <= tol ||b|| (or at the iteration cap; the true residual is
-// checked afterwards), else beta = rr / rho and rho = rr.
-SEED_DEV void cg_update_tail(const CgCols &c, int col, double rr) {
-  const double rn = sqrt(rr), bn = c.bnorm[col];
-  c.iters[col] += 1;
-  c.mvps[col] += 1;
-  c.relres[col] = bn > 0.0 ? rn / bn : 0.0;
-  if (rn <= c.tol * bn) {
+// Lockstep CG, after r -= alpha q and rr = ||r||^2, in the block that reduced column
+// col: count the iteration, stop the column when ||r|| <= tol ||b|| (or at the
+// iteration cap; the true residual is checked afterwards), else beta = rr / rho and
+// rho = rr.  The column's state is loaded before the partial sums are added up
+// (CgState: its round trip to L2 overlaps theirs), and the first warp forms the
+// two quotients, beta and the relative residual, side by side in two lanes: what
+// follows the last block's arrival is latency of the whole iteration.
+struct CgState {
+  double bn, rho;
+  int32_t iters, mvps;
+};
+SEED_DEV CgState cg_state(const CgCols &c, int col) {
+  return CgState{__ldcg(c.bnorm + col), __ldcg(c.rho + col), __ldcg(c.iters + col), __ldcg(c.mvps + col)};
+}
+SEED_DEV void cg_update_tail(const CgCols &c, int col, double rr, const CgState &t) {   // the first warp
+  if (threadIdx.x >= 32) return;
+  const double rn = sqrt(rr);
+  const double quot = (threadIdx.x == 1 ? rn : rr) / (threadIdx.x == 1 ? t.bn : t.rho);
+  const double rel = __shfl_sync(0xffffffffu, quot, 1);
+  if (threadIdx.x != 0) return;
+  c.iters[col] = t.iters + 1;
+  c.mvps[col] = t.mvps + 1;
+  c.relres[col] = t.bn > 0.0 ? rel : 0.0;
+  if (rn <= c.tol * t.bn) {
     c.active[col] = 0;
     c.reached[col] = 1;
     c.needs_check[col] = 1;
-  } else if (c.iters[col] >= c.maxit || !isfinite(rr)) {
+  } else if (t.iters + 1 >= c.maxit || !isfinite(rr)) {
     // a NaN or infinite residual (non-finite input, or p^H A p <= 0 on an
     // operator that is not positive definite) ends the column unconverged
     c.active[col] = 0;
     c.needs_check[col] = 1;
   } else {
-    c.beta[col] = rr / c.rho[col];
+    c.beta[col] = quot;
     c.rho[col] = rr;
   }
 }

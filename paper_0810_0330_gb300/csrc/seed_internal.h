@@ -148,11 +148,12 @@ struct CgCols {
   int32_t nc;
   double *rho, *alpha, *beta, *bnorm, *relres, *rupd;
   int32_t *active, *iters, *reached, *restarts, *converged, *needs_check, *mvps, *upd;
+  int32_t *stepped;   // the column took part in the current iteration (its x update is still to come)
   double tol, tol_check, delta;
   int32_t maxit, max_restarts;
 };
 constexpr int kCgDoubles = 6;   // arrays of kMaxRhs doubles in CgCols
-constexpr int kCgInts = 8;      // arrays of kMaxRhs int32 in CgCols
+constexpr int kCgInts = 9;      // arrays of kMaxRhs int32 in CgCols
 
 // Grid barrier of the persistent kernels (all zeroed before every launch).
 constexpr int kGridSyncWords = 4 + 256;
@@ -167,6 +168,18 @@ struct GridSync {
 // ---------------------------------------------------------------------------
 // launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
+
+// Lockstep CG's alpha[col] = rho[col] / Re(p^H q), formed by the kernel that writes q = A p (P:
+// columns as far apart as q's; part: partial sums, one per block or warp and column; tickets as
+// CgCols' reductions).
+template <class T>
+struct CgDot {
+  const T *P;
+  double *part;
+  unsigned *tickets;
+  const double *rho;
+  double *alpha;
+};
 
 // Wilson-Dirac (wilson.cu).  sign = +1 applies D, -1 applies D^H.
 // C = double2 (FP64 links) or float2 (FP32 copy of the links, mixed precision)
@@ -188,7 +201,8 @@ void launch_wilson_dslash(const WilsonOp &op, int sign, const double2 *in, int64
 // spinor vectors use the mixed path's 32-site tiled layout (Layout32), else the
 // caller's site-major layout.
 void launch_wilson_dslash32(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, float2 *out, int64_t ldo,
-                            int ncols, const int32_t *col_active, bool tiled, cudaStream_t s);
+                            int ncols, const int32_t *col_active, bool tiled, cudaStream_t s,
+                            const CgDot<float2> *dot = nullptr);   // dot: tiled only
 void launch_links_soa32(const double2 *links, float2 *out, int64_t sites, cudaStream_t s);
 
 // The FP64 operator in fixed-point arithmetic (wilson_fixed.cuh): WilsonOp plus
@@ -209,19 +223,10 @@ void launch_fix_spinors(const WilsonFix &op, const double2 *X, int64_t ldx, int4
                         int ncols, const int32_t *col_active, cudaStream_t s);
 // few enough tiles x columns for the form with one warp per direction and half-spinor component
 bool fix_few(int64_t sites, int ncols);
-// lockstep CG's alpha[col] = rho[col] / Re(P^H out), formed with the last operator half
-// (P: ldo apart; part: ceil(sites / 16) doubles per column; tickets as CgCols' reductions)
-struct FixDot {
-  const double2 *P;
-  double *part;
-  unsigned *tickets;
-  const double *rho;
-  double *alpha;
-};
 // (q, e) -> (qout, eout), or -> out (doubles, site-major, ldo) when qout is NULL; dot: with D^H only
 void launch_dslash_fix(const WilsonFix &op, int sign, const int4 *in, const int32_t *ein, int64_t ldq, int4 *qout,
                        int32_t *eout, double2 *out, int64_t ldo, int ncols, const int32_t *col_active,
-                       cudaStream_t s, const FixDot *dot = nullptr);
+                       cudaStream_t s, const CgDot<double2> *dot = nullptr);
 
 // CSR (csr.cu)
 template <class R>
@@ -263,10 +268,14 @@ template <class T> void launch_cg_alpha(int64_t n, const T *P, const T *Q, int64
                                         double *partials, unsigned *tickets, cudaStream_t s);
 template <class T> void launch_cg_update(int64_t n, const CallArgs *call, T *R, const T *P, const T *Q, int64_t ld,
                                          const CgCols &c, double *partials, unsigned *tickets, cudaStream_t s);
-// The Wilson CG's form: r and its norm only (X untouched), sets upd[col] for launch_cg_xp_fix
-void launch_cg_residual(int64_t n, double2 *R, const double2 *Q, int64_t ld, const CgCols &c, double *partials,
-                        unsigned *tickets, cudaStream_t s);
-// x += alpha p, p = r + beta p and p's blocks (q, e), columns with upd set
+// The lockstep CG's iteration after q and alpha: r -= alpha q with the column's norm, test and beta,
+// setting stepped[col]; then, for the columns with stepped set, x += alpha p and (still
+// active) p = r + beta p.
+template <class T> void launch_cg_residual(int64_t n, T *R, const T *Q, int64_t ld, const CgCols &c, double *partials,
+                                           unsigned *tickets, cudaStream_t s);
+template <class T> void launch_cg_xp(int64_t n, const CallArgs *call, const T *R, T *P, int64_t ld, const CgCols &c,
+                                     cudaStream_t s);
+// the same with p's fixed-point blocks (q, e)
 void launch_cg_xp_fix(const WilsonFix &op, const CallArgs *call, const double2 *R, double2 *P, int64_t ld, int4 *q,
                       int32_t *e, const CgCols &c, cudaStream_t s);
 template <class T> void launch_cg_p(int64_t n, const T *R, T *P, int64_t ld, const CgCols &c, cudaStream_t s);

@@ -73,11 +73,26 @@ SEED_DEV void hops32(const float2 *__restrict__ in, int32_t nf, int32_t nb, cons
   hop_pair_r<MU, S>(pf, uf, negf, pb, ub, negb, acc);
 }
 
-template <int S, bool VEC, bool TILED>
+// Lockstep CG's alpha of column c from the blocks' partial sums of p^H q (FP32 per thread, FP64
+// above), in block order by the column's last of nb blocks; block: this block's place.
+SEED_DEV void dot32(float pq, int c, int64_t block, int nb, const CgDot<float2> &dot, double *sm) {
+  double v[1] = {(double)pq};
+  block_sum<1, 128>(v, sm);
+  double *part = dot.part + (int64_t)c * nb;
+  if (threadIdx.x == 0) part[block] = v[0];
+  if (!last_block_done(dot.tickets + kColTicket + c, (unsigned)nb)) return;
+  const double rho = __ldcg(dot.rho + c);
+  const double t = sum_partials<128>(part, nb, 1, 0, sm);
+  if (threadIdx.x == 0) dot.alpha[c] = rho / t;
+}
+
+template <int S, bool VEC, bool TILED, bool DOT = false>
 __global__ void __launch_bounds__(128) k_dslash32(WilsonOp32 op, const float2 *__restrict__ in, int64_t ldi,
                                                   float2 *__restrict__ out, int64_t ldo,
-                                                  const int32_t *__restrict__ col_active, int ncols, int group) {
+                                                  const int32_t *__restrict__ col_active, int ncols, int group,
+                                                  CgDot<float2> dot) {
   __shared__ float sacc[4][24][kWilsonSites + 1];
+  __shared__ double sm[4];
   const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
   const int64_t s0 = (int64_t)blockIdx.x * kWilsonSites;
   const int64_t s = s0 + lane;
@@ -129,7 +144,11 @@ __global__ void __launch_bounds__(128) k_dslash32(WilsonOp32 op, const float2 *_
     if constexpr (TILED) {
       // this block's tile: 768 contiguous floats, component k at [64 k, 64 k + 64)
       const int64_t base = (s0 >> 5) * 768;
-      for (int o = threadIdx.x; o < 768; o += 128) {
+      const float *pd = DOT ? reinterpret_cast<const float *>(dot.P + (int64_t)c * ldo) : nullptr;
+      float pq = 0.f;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        const int o = threadIdx.x + 128 * q;
         const int k = o >> 6, rem = o & 63, sl = rem >> 1, cc = 2 * k + (rem & 1);
         float v = 0.f;   // padding sites stay zero
         if (s0 + sl < op.sites) {
@@ -137,7 +156,9 @@ __global__ void __launch_bounds__(128) k_dslash32(WilsonOp32 op, const float2 *_
           v = fmaf(mk, sum, __ldg(ind + base + o));
         }
         outd[base + o] = v;
+        if constexpr (DOT) pq = fmaf(__ldg(pd + base + o), v, pq);
       }
+      if constexpr (DOT) dot32(pq, c, blockIdx.x, gridDim.x, dot, sm);
     } else {
       for (int o = threadIdx.x; o < kWilsonSites * 24; o += 128) {
         const int sl = o / 24, cc = o - 24 * (o / 24);
@@ -213,10 +234,11 @@ SEED_DEV void site_dir2(const WilsonOp32 &op, const float2 *__restrict__ in, int
 
 // Grid: one block per (128 sites, column pair), the pair fastest, so that the
 // pairs of one site block run together and their link loads hit L2.
-template <int S, bool TILED, bool VEC>
+template <int S, bool TILED, bool VEC, bool DOT = false>
 __global__ void __launch_bounds__(128, 4) k_dslash32_site(WilsonOp32 op, const float2 *__restrict__ in, int64_t ldi,
                                                           float2 *__restrict__ out, int64_t ldo,
-                                                          const int32_t *__restrict__ col_active, int ncols) {
+                                                          const int32_t *__restrict__ col_active, int ncols,
+                                                          CgDot<float2> dot) {
   const int npairs = (ncols + 1) / 2;
   const int64_t sblock = (int64_t)blockIdx.x / npairs;
   const int c0 = 2 * (int)(blockIdx.x - sblock * npairs);
@@ -227,7 +249,8 @@ __global__ void __launch_bounds__(128, 4) k_dslash32_site(WilsonOp32 op, const f
   if (jm == 0u) return;   // uniform over the block
   const int64_t s = sblock * 128 + threadIdx.x;
   const int64_t send = TILED ? (op.sites + 31) / 32 * 32 : op.sites;
-  if (s >= send) return;
+  const bool write = s < send;
+  if (!DOT && !write) return;
   const bool valid = s < op.sites;   // tiled padding sites only write zeros
   in += (int64_t)c0 * ldi;
   out += (int64_t)c0 * ldo;
@@ -254,14 +277,23 @@ __global__ void __launch_bounds__(128, 4) k_dslash32_site(WilsonOp32 op, const f
     if (!(jm & (1u << j))) continue;
     const float2 *ic = in + j * ldi + so;
     float2 *oc = out + j * ldo + so;
+    float pq = 0.f;
+    if (write) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      float2 v = make_float2(0.f, 0.f);
-      if (valid) {
-        const float2 x = __ldg(ic + kStride * k);
-        v = make_float2(fmaf(mk, acc[j][k].x, x.x), fmaf(mk, acc[j][k].y, x.y));
+      for (int k = 0; k < 12; ++k) {
+        float2 v = make_float2(0.f, 0.f);
+        if (valid) {
+          const float2 x = __ldg(ic + kStride * k);
+          v = make_float2(fmaf(mk, acc[j][k].x, x.x), fmaf(mk, acc[j][k].y, x.y));
+          if constexpr (DOT)
+            pq = Sc<float2>::redot(__ldg(dot.P + (int64_t)(c0 + j) * ldo + so + kStride * k), v, pq);
+        }
+        __stcs(oc + kStride * k, v);   // streaming store: this kernel does not read it again
       }
-      __stcs(oc + kStride * k, v);   // streaming store: this kernel does not read it again
+    }
+    if constexpr (DOT) {
+      __shared__ double sm[4];
+      dot32(pq, c0 + j, sblock, gridDim.x / npairs, dot, sm);
     }
   }
 }
@@ -285,7 +317,7 @@ void launch_links_soa32(const double2 *links, float2 *out, int64_t sites, cudaSt
 // Column groups: enough blocks to give every SM about four, otherwise all
 // columns of a site block in one group (links read once).
 void launch_wilson_dslash32(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, float2 *out, int64_t ldo,
-                            int ncols, const int32_t *col_active, bool tiled, cudaStream_t s) {
+                            int ncols, const int32_t *col_active, bool tiled, cudaStream_t s, const CgDot<float2> *dot) {
   const int64_t nsb = (op.sites + kWilsonSites - 1) / kWilsonSites;
   int64_t group = (nsb * ncols) / (152 * 4);
   if (group < 1) group = 1;
@@ -293,31 +325,36 @@ void launch_wilson_dslash32(const WilsonOp32 &op, int sign, const float2 *in, in
   const int ngroups = (int)((ncols + group - 1) / group);
   const dim3 grid((unsigned)nsb, (unsigned)ngroups);
   const bool vec = ((uintptr_t)in % 16 == 0) && (ldi % 2 == 0);
+  const CgDot<float2> d = dot ? *dot : CgDot<float2>{};
   if (op.sites >= kSiteKernelSites) {
     const int64_t nthreads = tiled ? nsb * kWilsonSites : op.sites;
     const unsigned g2 = (unsigned)(((nthreads + 127) / 128) * ((ncols + 1) / 2));
-    if (tiled) {
-      if (sign > 0) k_dslash32_site<+1, true, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
-      else k_dslash32_site<-1, true, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
+    if (dot != nullptr) {   // lockstep CG: q = D^H t with alpha
+      k_dslash32_site<-1, true, false, true><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
+    } else if (tiled) {
+      if (sign > 0) k_dslash32_site<+1, true, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
+      else k_dslash32_site<-1, true, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
     } else if (vec) {
-      if (sign > 0) k_dslash32_site<+1, false, true><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
-      else k_dslash32_site<-1, false, true><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
+      if (sign > 0) k_dslash32_site<+1, false, true><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
+      else k_dslash32_site<-1, false, true><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
     } else {
-      if (sign > 0) k_dslash32_site<+1, false, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
-      else k_dslash32_site<-1, false, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols);
+      if (sign > 0) k_dslash32_site<+1, false, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
+      else k_dslash32_site<-1, false, false><<<g2, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, d);
     }
     return;
   }
   const int g = (int)group;
-  if (tiled) {
-    if (sign > 0) k_dslash32<+1, false, true><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
-    else k_dslash32<-1, false, true><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
+  if (dot != nullptr) {
+    k_dslash32<-1, false, true, true><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
+  } else if (tiled) {
+    if (sign > 0) k_dslash32<+1, false, true><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
+    else k_dslash32<-1, false, true><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
   } else if (sign > 0) {
-    if (vec) k_dslash32<+1, true, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
-    else k_dslash32<+1, false, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
+    if (vec) k_dslash32<+1, true, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
+    else k_dslash32<+1, false, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
   } else {
-    if (vec) k_dslash32<-1, true, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
-    else k_dslash32<-1, false, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g);
+    if (vec) k_dslash32<-1, true, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
+    else k_dslash32<-1, false, false><<<grid, 128, 0, s>>>(op, in, ldi, out, ldo, col_active, ncols, g, d);
   }
 }
 

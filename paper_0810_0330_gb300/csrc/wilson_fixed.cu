@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(FT, 3) k_dslash_fix(WilsonFix op, const int4 *
                                                       const int32_t *__restrict__ ein, int64_t ldq,
                                                       int4 *__restrict__ qout, int32_t *__restrict__ eout,
                                                       double2 *__restrict__ out, int64_t ldo, int64_t items, int ncols,
-                                                      const int32_t *__restrict__ col_active, FixDot dot) {
+                                                      const int32_t *__restrict__ col_active, CgDot<double2> dot) {
   extern __shared__ double stage_all[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, sl = lane & 15;
   const int64_t item = (int64_t)blockIdx.x * (FT / 32) + warp;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(DT, 3) k_dslash_fix_dir(WilsonFix op, const in
                                                           const int32_t *__restrict__ ein, int64_t ldq,
                                                           int4 *__restrict__ qout, int32_t *__restrict__ eout,
                                                           double2 *__restrict__ out, int64_t ldo, int ncols,
-                                                          const int32_t *__restrict__ col_active, FixDot dot) {
+                                                          const int32_t *__restrict__ col_active, CgDot<double2> dot) {
   __shared__ long long sacc[4][2][12][32];   // [direction][component][up, low reals][site]
   __shared__ int sE[4][32];
   __shared__ unsigned sO[4][2][32];
@@ -486,8 +486,9 @@ __global__ void __launch_bounds__(DT, 3) k_dslash_fix_dir(WilsonFix op, const in
       block_sum<1, DT>(t, sred);
       if (threadIdx.x == 0) part[tile] = t[0];
       if (!last_block_done(dot.tickets + kColTicket + col, (unsigned)tiles)) return;
+      const double rho = __ldcg(dot.rho + col);
       const double sum = sum_partials<DT>(part, tiles, 1, 0, sred);
-      if (threadIdx.x == 0) dot.alpha[col] = dot.rho[col] / sum;
+      if (threadIdx.x == 0) dot.alpha[col] = rho / sum;
     }
   }
 }
@@ -499,11 +500,11 @@ bool fix_few(int64_t sites, int ncols) { return (sites + 31) / 32 * ncols <= kFi
 
 void launch_dslash_fix(const WilsonFix &op, int sign, const int4 *in, const int32_t *ein, int64_t ldq, int4 *qout,
                        int32_t *eout, double2 *out, int64_t ldo, int ncols, const int32_t *col_active, cudaStream_t s,
-                       const FixDot *dot) {
+                       const CgDot<double2> *dot) {
   if (ncols < 1) return;
   const int64_t items = (op.sites + 15) / 16 * ncols;
   const unsigned grid = (unsigned)((items + FT / 32 - 1) / (FT / 32));
-  const FixDot d = dot ? *dot : FixDot{};
+  const CgDot<double2> d = dot ? *dot : CgDot<double2>{};
   const int64_t tiles = (op.sites + 31) / 32;
 #define FIX_GO(S, OUT)                                                                                              \
   if (fix_few(op.sites, ncols))                                                                                     \
@@ -531,7 +532,7 @@ void launch_dslash_fix(const WilsonFix &op, int sign, const int4 *in, const int3
 // ---------------------------------------------------------------------------
 // Lockstep CG, end of an iteration: x += alpha p (deferred to here from the
 // residual's update, so that p is read once), p = r + beta p, and p's blocks for
-// the next D.  A column that has just stopped (upd set, not active) takes its x
+// the next D.  A column that has just stopped (stepped set, not active) takes its x
 // update only.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(CT) k_cg_xp_fix(const CallArgs *call, const double2 *__restrict__ R,
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(CT) k_cg_xp_fix(const CallArgs *call, const do
   __shared__ double st[32 * kFixPitch];
   const int64_t tile = blockIdx.x / c.nc;
   const int col = (int)(blockIdx.x - tile * c.nc);
-  if (!c.upd[col]) return;
+  if (!c.stepped[col]) return;
   const bool act = c.active[col] != 0;
   const double al = c.alpha[col], be = c.beta[col];
   double2 *x = reinterpret_cast<double2 *>(call->X) + (int64_t)(col + call->col0) * call->ldx + tile * 384;
