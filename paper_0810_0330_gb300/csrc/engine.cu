@@ -387,18 +387,35 @@ int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int
   return 3;
 }
 
-// Y = A X with the FP32 copy of the operator (mixed precision).  Returns the kernel count.
-// tiled: X and Y in the solver's tiled FP32 layout (else the caller's site-major one).
-int apply_A32(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, const int32_t *mask,
-              bool tiled = true) {
+// Y = op X with the FP32 copy of the operator (mixed precision), op 0 = A, 1 = D, 2 = D^H.
+// tiled: X and Y in the solver's tiled FP32 layout (else the caller's site-major one; on large
+// lattices that goes through tiled columns in P32 and T32).  Returns the kernel count.
+int apply_32(seed_ctx *ctx, int op, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, bool tiled) {
   if (ctx->kind == 0) {
-    launch_csr_spmv32(ctx->csr32, (const float *)X, ldx, (float *)Y, ldy, ncols, mask, ctx->cs);
+    launch_csr_spmv32(ctx->csr32, (const float *)X, ldx, (float *)Y, ldy, ncols, nullptr, ctx->cs);
     return 1;
   }
-  launch_wilson_dslash32(ctx->wil32, +1, (const float2 *)X, ldx, (float2 *)ctx->T32, ctx->ldv, ncols, mask, tiled,
-                         ctx->cs);
-  launch_wilson_dslash32(ctx->wil32, -1, (const float2 *)ctx->T32, ctx->ldv, (float2 *)Y, ldy, ncols, mask, tiled,
-                         ctx->cs);
+  const WilsonOp32 &w = ctx->wil32;
+  const float2 *x = (const float2 *)X;
+  float2 *y = (float2 *)Y, *t = (float2 *)ctx->T32;
+  const int64_t ld = ctx->ldv;
+  if (!tiled && dslash32_tiles(w.sites)) {
+    float2 *p = (float2 *)ctx->P32;
+    launch_tile32(x, ldx, p, ld, w.sites, ncols, ctx->cs);
+    if (op != 0) {
+      launch_wilson_dslash32_user(w, op == 1 ? +1 : -1, p, ld, y, ldy, ncols, ctx->cs);
+      return 2;
+    }
+    launch_wilson_dslash32(w, +1, p, ld, t, ld, ncols, nullptr, true, ctx->cs);
+    launch_wilson_dslash32_user(w, -1, t, ld, y, ldy, ncols, ctx->cs);
+    return 3;
+  }
+  if (op != 0) {
+    launch_wilson_dslash32(w, op == 1 ? +1 : -1, x, ldx, y, ldy, ncols, nullptr, tiled, ctx->cs);
+    return 1;
+  }
+  launch_wilson_dslash32(w, +1, x, ldx, t, ld, ncols, nullptr, tiled, ctx->cs);
+  launch_wilson_dslash32(w, -1, t, ld, y, ldy, ncols, nullptr, tiled, ctx->cs);
   return 2;
 }
 
@@ -501,7 +518,7 @@ template <class T>
 int issue_seed_step(seed_ctx *ctx, int nrhs, bool reorth) {
   SeedBufs<T> b = seed_bufs<T>(ctx, nrhs);
   // u = A f with f = beta_{i-1} v_i not yet normalized: the dots kernel forms v_i and scales u
-  int k = kLow<T> ? apply_A32(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1, nullptr)
+  int k = kLow<T> ? apply_32(ctx, 0, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1, true)
                   : apply_A64(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1);
   launch_seed_dots<T>(b, ctx->cs);
   launch_seed_update<T>(b, !reorth, ctx->cs);
@@ -2028,11 +2045,9 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   StreamScope scope(ctx);
   if (op == 0 && fix_pays(ctx, ncols)) TRY(ensure_fixed(ctx));
   if (op == 3) {
-    ctx->stats.kernel_launches += apply_A32(ctx, X, ldx, Y, ldy, ncols, nullptr, false);
+    ctx->stats.kernel_launches += apply_32(ctx, 0, X, ldx, Y, ldy, ncols, false);
   } else if (op >= 4) {
-    launch_wilson_dslash32(ctx->wil32, (op == 4 || op == 6) ? +1 : -1, (const float2 *)X, ldx, (float2 *)Y, ldy,
-                           ncols, nullptr, tiled, ctx->cs);
-    ctx->stats.kernel_launches += 1;
+    ctx->stats.kernel_launches += apply_32(ctx, (op == 4 || op == 6) ? 1 : 2, X, ldx, Y, ldy, ncols, tiled);
   } else if (op == 0) {
     ctx->stats.kernel_launches += apply_A(ctx, X, ldx, Y, ldy, ncols, nullptr);
     ctx->stats.mvps += ncols;
@@ -2145,7 +2160,7 @@ seed_status seed_time_operator(seed_ctx *ctx, int32_t op, int32_t ncols, int32_t
     if (op == 0) {
       ctx->stats.kernel_launches += apply_A(ctx, ctx->P, ctx->ldv, ctx->Q, ctx->ldv, ncols, nullptr);
     } else if (op == 3) {
-      ctx->stats.kernel_launches += apply_A32(ctx, ctx->P32, ctx->ldv, ctx->Q32, ctx->ldv, ncols, nullptr);
+      ctx->stats.kernel_launches += apply_32(ctx, 0, ctx->P32, ctx->ldv, ctx->Q32, ctx->ldv, ncols, true);
     } else if (op >= 4) {
       launch_wilson_dslash32(ctx->wil32, op == 4 ? +1 : -1, (const float2 *)ctx->P32, ctx->ldv, (float2 *)ctx->Q32,
                              ctx->ldv, ncols, nullptr, true, ctx->cs);

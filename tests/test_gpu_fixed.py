@@ -180,3 +180,31 @@ def test_links_changed_in_place(seedlib):
     ref = on_gpu(seedlib, dims, kappa, 0, U2, x, 0)
     assert np.array_equal(Y.t().cpu().numpy(), ref)
     seedlib.seed_destroy(ctx)
+
+
+def test_fp32_operator_on_the_callers_layout_ragged(seedlib, orc):
+    """FP32 operator from 65536 sites on (tiled through work space): a partial last
+    tile and block, an odd column count, a leading dimension above n; the FP32 bound of test_gpu_mixed."""
+    from paper_0810_0330_gb300 import inputs as I
+    import torch
+    dims, kappa = (17, 15, 17, 16), 0.155
+    vol = int(np.prod(dims))
+    n = 12 * vol
+    rng = np.random.default_rng(4)
+    U = I.random_su3_links(dims, 0.3, seed=5)
+    ctx = seedlib.seed_create_wilson(dims, kappa, torch.from_numpy(U).cuda(),
+                                     seedlib.seed_params_default(m_max=2, precision=1), bc_t=1)
+    x = (rng.standard_normal((3, n + 5)) + 1j * rng.standard_normal((3, n + 5))).astype(np.complex64)
+    buf = torch.from_numpy(x).cuda()
+    for op, sign in ((3, 0), (4, 1), (5, -1)):
+        y = torch.full((3, n + 7), 7.0, dtype=torch.complex64, device="cuda")
+        seedlib.seed_apply(ctx, op, buf[:, :n].t(), y[:, :n].t())
+        got = y.cpu().numpy()
+        assert np.all(got[:, n:] == 7.0)   # nothing past the column's end
+        v = x[2, :n].astype(np.complex128)
+        if sign == 0:
+            ref = orc.wilson_dslash(dims, kappa, 1, -1, U, orc.wilson_dslash(dims, kappa, 1, 1, U, v))
+        else:
+            ref = orc.wilson_dslash(dims, kappa, 1, sign, U, v)
+        assert np.linalg.norm(got[2, :n] - ref) <= 1e-6 * np.linalg.norm(ref)
+    seedlib.seed_destroy(ctx)
