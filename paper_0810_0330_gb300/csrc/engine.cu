@@ -352,9 +352,14 @@ seed_status ensure_fixed(seed_ctx *ctx) {
 int4 *fix_T(seed_ctx *ctx) { return reinterpret_cast<int4 *>(ctx->T); }
 int32_t *fix_Te(seed_ctx *ctx) { return ctx->Fe + ctx->ldv / 12 * ctx->cap_cols; }
 
-// Y = A X on ncols columns in FP64 arithmetic throughout.  The Lanczos steps of the seed system take
-// this form: they amplify a last-bit change of A v_i until the late basis vectors, and through
-// the Galerkin projection the error (not the size) of the seeded solutions, differ by a per cent.
+// Y = A X on ncols columns in FP64 arithmetic throughout.  On small lattices the Lanczos steps of the
+// seed system take this form: they amplify a last-bit change of A v_i until the late basis
+// vectors, and through the Galerkin projection the error (not the size) of the seeded
+// solutions, differ by a per cent.  Measured as the change of x^2.. (12 point sources, CG to 1e-8)
+// when b changes in its last bit: 3e-10 to 1e-9 on 6 x 8^3, 8^4 and 8^3 x 12, 4e-13 on 8^3
+// x 16, 5e-14 on 12^4 and below 1e-13 on 16^4; so from kFixSeedSites on they take the
+// fixed-point operator (apply_seed).
+constexpr int64_t kFixSeedSites = 16384;
 int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols) {
   if (ctx->kind == 0) {
     launch_csr_spmv(ctx->csr, (const double *)X, ldx, (double *)Y, ldy, ncols, nullptr, ctx->cs);
@@ -368,6 +373,7 @@ int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, i
 // Y = A X on ncols columns (mask: skip columns whose flag is 0).  Returns the kernel count.
 // Wilson: in fixed-point arithmetic from one tile per SM on; below that the FP64 kernel's two
 // launches (7 us each, one tile's FP64 instructions on its SM) are the shorter chain.
+bool fix_seed(const seed_ctx *ctx) { return ctx->kind == 1 && ctx->wfix.sites >= kFixSeedSites; }
 bool fix_pays(const seed_ctx *ctx, int ncols) { return ctx->kind == 1 && ctx->ldv / 384 * ncols > ctx->sm_count; }
 int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, const int32_t *mask) {
   if (ctx->kind == 0) {
@@ -385,6 +391,11 @@ int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int
   launch_dslash_fix(ctx->wfix, -1, fix_T(ctx), fix_Te(ctx), ld, nullptr, nullptr, (double2 *)Y, ldy, ncols, mask,
                     ctx->cs);
   return 3;
+}
+
+// Y = A X where the result feeds the seed recurrence
+int apply_seed(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols) {
+  return fix_seed(ctx) ? apply_A(ctx, X, ldx, Y, ldy, ncols, nullptr) : apply_A64(ctx, X, ldx, Y, ldy, ncols);
 }
 
 // Y = op X with the FP32 copy of the operator (mixed precision), op 0 = A, 1 = D, 2 = D^H.
@@ -519,7 +530,7 @@ int issue_seed_step(seed_ctx *ctx, int nrhs, bool reorth) {
   SeedBufs<T> b = seed_bufs<T>(ctx, nrhs);
   // u = A f with f = beta_{i-1} v_i not yet normalized: the dots kernel forms v_i and scales u
   int k = kLow<T> ? apply_32(ctx, 0, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1, true)
-                  : apply_A64(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1);
+                  : apply_seed(ctx, ctx->f, ctx->ldv, ctx->u, ctx->ldv, 1);
   launch_seed_dots<T>(b, ctx->cs);
   launch_seed_update<T>(b, !reorth, ctx->cs);
   k += 2;
@@ -577,10 +588,12 @@ int csr_seed_grid(const seed_ctx *ctx) {
 // The Wilson runs take their resident form when the lattice has no more
 // 32-site tiles than blocks, else the general one (FP32: the site form, one
 // thread per site; 16^3 x 32 mixed seed phase 40.1 ms from graphs of step
-// kernels, 37.1 ms in the site form).
+// kernels, 37.1 ms in the site form).  Not in FP64 from kFixSeedSites on: there
+// step kernels with the fixed-point operator beat the run's FP64 tiles (16^4, 303
+// steps: 176 -> 95 ms).
 bool use_persistent_seed(seed_ctx *ctx) {
   const int f = ctx->prm.reorth_freq;
-  return ctx->allow_persistent && ctx->pgrid > 0 && (f == 0 || f >= 8);
+  return ctx->allow_persistent && ctx->pgrid > 0 && (f == 0 || f >= 8) && !(ctx->precision == 0 && fix_seed(ctx));
 }
 
 // Blocks of the persistent CSR CG: one per work item (1024 rows of one column)
@@ -762,7 +775,7 @@ seed_status solve_first_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
     if (nrhs > 1) launch_copy_cols<T>((const T *)B + ldb, ldb, (T *)ctx->R, ctx->ldv, n, nrhs - 1, ctx->cs);
     kern += 1 + (nrhs > 1);
   } else {
-    kern += apply_A64(ctx, X, ldx, ctx->Q, ctx->ldv, nrhs);
+    kern += apply_seed(ctx, X, ldx, ctx->Q, ctx->ldv, nrhs);
     ctx->stats.mvps += nrhs;
     launch_sub_from<T>((const T *)B, ldb, (const T *)ctx->Q, ctx->ldv, (T *)ctx->P, ctx->ldv, n, nrhs, ctx->cs);
     if (nrhs > 1) launch_copy_cols<T>((const T *)ctx->P + ctx->ldv, ctx->ldv, (T *)ctx->R, ctx->ldv, n, nrhs - 1, ctx->cs);
@@ -2043,7 +2056,7 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   if (overlap(X, ldx, Y, ldy, ncols, len, es)) return fail(ctx, SEED_EINVAL, "X and Y overlap");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
-  if (op == 0 && fix_pays(ctx, ncols)) TRY(ensure_fixed(ctx));
+  if (op < 3 && (op == 0 ? fix_pays(ctx, ncols) : fix_seed(ctx))) TRY(ensure_fixed(ctx));
   if (op == 3) {
     ctx->stats.kernel_launches += apply_32(ctx, 0, X, ldx, Y, ldy, ncols, false);
   } else if (op >= 4) {
@@ -2052,7 +2065,15 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
     ctx->stats.kernel_launches += apply_A(ctx, X, ldx, Y, ldy, ncols, nullptr);
     ctx->stats.mvps += ncols;
   } else {
-    // D and D^H by themselves form right-hand sides of the seed system (b = D^H eta): FP64, see apply_A64
+    // D and D^H by themselves form right-hand sides of the seed system (b = D^H eta): as apply_seed
+    if (fix_seed(ctx)) {
+      launch_fix_spinors(ctx->wfix, (const double2 *)X, ldx, ctx->F, ctx->ldv, ctx->Fe, ncols, nullptr, ctx->cs);
+      launch_dslash_fix(ctx->wfix, op == 1 ? +1 : -1, ctx->F, ctx->Fe, ctx->ldv, nullptr, nullptr, (double2 *)Y, ldy,
+                        ncols, nullptr, ctx->cs);
+      ctx->stats.kernel_launches += 2;
+      CU(cudaGetLastError());
+      return SEED_OK;
+    }
     launch_wilson_dslash(ctx->wil, op == 1 ? +1 : -1, (const double2 *)X, ldx, (double2 *)Y, ldy, ncols, nullptr,
                          ctx->cs);
     ctx->stats.kernel_launches += 1;

@@ -182,6 +182,32 @@ def test_links_changed_in_place(seedlib):
     seedlib.seed_destroy(ctx)
 
 
+def test_seed_steps_on_a_large_lattice(seedlib, orc):
+    """From 16384 sites on the FP64 seed run takes step kernels with the fixed-point operator:
+    D and D^H by themselves and the whole solve against the oracle, as in the parity tests."""
+    from paper_0810_0330_gb300 import inputs as I
+    from test_gpu_parity import REL_X, compare_full, dev_cols, host_cols, relerr, run_gpu, self_sensitivity, wilson_ctx
+    import torch
+    dims, kappa = (8, 16, 8, 16), 0.12
+    U = I.random_su3_links(dims, 0.3, seed=2)
+    B = I.gaussian_rhs(12 * 16384, 2, seed=3, complex_=True)
+    kw = dict(m_max=200, reorth_freq=25)
+    ctx = wilson_ctx(seedlib, dims, kappa, U, bc_t=1, tol_seed=1e-10, tol_rest=1e-8, **kw)
+    for op_, sign in ((1, 1), (2, -1)):
+        X = dev_cols(B)
+        Y = torch.empty_like(X.t()).t()
+        seedlib.seed_apply(ctx, op_, X, Y)
+        ref = orc.wilson_dslash(dims, kappa, 1, sign, U, B[:, 1])
+        assert relerr(host_cols(Y)[:, 1], ref) < 1e-15 * 4
+    info1, info2, Xs, X = run_gpu(seedlib, ctx, B)
+    op = orc.Operator.wilson(dims, kappa, U, bc_t=1)
+    ref = orc.seed_solve_all(op, B, tol_seed=1e-10, tol_rest=1e-8, **kw)
+    s_seed, s_final = self_sensitivity(orc, op, B, ref, cols=(1,), tol=1e-10, **kw)
+    compare_full(ref, info1, info2, Xs, X, "wilson-large", seeded_tol=max(REL_X, 10 * s_seed),
+                 final_tol=max(REL_X, 10 * s_final))
+    seedlib.seed_destroy(ctx)
+
+
 def test_fp32_operator_on_the_callers_layout_ragged(seedlib, orc):
     """FP32 operator from 65536 sites on (tiled through work space): a partial last
     tile and block, an odd column count, a leading dimension above n; the FP32 bound of test_gpu_mixed."""
