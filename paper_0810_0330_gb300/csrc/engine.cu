@@ -336,16 +336,26 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
 // What the fixed-point operator needs, for a call that uses it (never inside a graph capture): its
 // work space for the context's columns, and the copy of the caller's links, once per call (the
 // caller may have changed them since the last one).
-seed_status ensure_fixed(seed_ctx *ctx) {
+seed_status ensure_fixed(seed_ctx *ctx, bool links = true) {
   if (ctx->kind != 1 || ctx->links_ready) return SEED_OK;
   const size_t cols = ctx->cap_cols;
   if (!ctx->F) TRY(dalloc(ctx, &ctx->F, (size_t)ctx->ldv * cols * sizeof(int4)));
   if (!ctx->Fe) TRY(dalloc(ctx, &ctx->Fe, sizeof(int32_t) * 2 * (size_t)(ctx->ldv / 12) * cols));
   if (!ctx->dotpart) TRY(dalloc(ctx, &ctx->dotpart, sizeof(double) * (size_t)(ctx->ldv / 192) * cols));
+  if (!links) return SEED_OK;
   launch_fix_links(ctx->wfix, ctx->cs);
   ctx->links_ready = true;
   ctx->stats.kernel_launches += 1;
   return SEED_OK;
+}
+
+// The same for the operator by itself: false (the caller takes the FP64 kernel, which needs no work
+// space) where an allocation fails or a capture of the caller's stream forbids it.
+bool try_fixed(seed_ctx *ctx, bool links) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (!ctx->F || !ctx->Fe || !ctx->dotpart)
+    if (cudaStreamIsCapturing(ctx->cs, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+  return ensure_fixed(ctx, links) == SEED_OK;
 }
 
 // T's columns hold blocks (16 bytes per component, like its doubles); Te: their exponents
@@ -372,7 +382,8 @@ int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, i
 
 // Y = A X on ncols columns (mask: skip columns whose flag is 0).  Returns the kernel count.
 // Wilson: in fixed-point arithmetic from one tile per SM on; below that the FP64 kernel's two
-// launches (7 us each, one tile's FP64 instructions on its SM) are the shorter chain.
+// launches (one tile's FP64 instructions on its SM) are the shorter chain than four, and
+// seed_apply converts links and spinors in one.
 bool fix_seed(const seed_ctx *ctx) { return ctx->kind == 1 && ctx->wfix.sites >= kFixSeedSites; }
 bool fix_pays(const seed_ctx *ctx, int ncols) { return ctx->kind == 1 && ctx->ldv / 384 * ncols > ctx->sm_count; }
 int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, const int32_t *mask) {
@@ -2056,17 +2067,26 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   if (overlap(X, ldx, Y, ldy, ncols, len, es)) return fail(ctx, SEED_EINVAL, "X and Y overlap");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
-  if (op < 3 && (op == 0 ? fix_pays(ctx, ncols) : fix_seed(ctx))) TRY(ensure_fixed(ctx));
+  const bool few = op == 0 && ctx->kind == 1 && !fix_pays(ctx, ncols);   // links and spinors converted in one launch
+  const bool fixed = ctx->kind == 1 && (op == 0 || (op < 3 && fix_seed(ctx))) && try_fixed(ctx, !few);
   if (op == 3) {
     ctx->stats.kernel_launches += apply_32(ctx, 0, X, ldx, Y, ldy, ncols, false);
   } else if (op >= 4) {
     ctx->stats.kernel_launches += apply_32(ctx, (op == 4 || op == 6) ? 1 : 2, X, ldx, Y, ldy, ncols, tiled);
+  } else if (few && fixed) {   // 4^4, one column: 24.6 -> 18.5 us a call (two FP64 launches before)
+    launch_fix_both(ctx->wfix, (const double2 *)X, ldx, ctx->F, ctx->ldv, ctx->Fe, ncols, ctx->cs);
+    launch_dslash_fix(ctx->wfix, +1, ctx->F, ctx->Fe, ctx->ldv, fix_T(ctx), fix_Te(ctx), nullptr, 0, ncols, nullptr,
+                      ctx->cs);
+    launch_dslash_fix(ctx->wfix, -1, fix_T(ctx), fix_Te(ctx), ctx->ldv, nullptr, nullptr, (double2 *)Y, ldy, ncols,
+                      nullptr, ctx->cs);
+    ctx->stats.kernel_launches += 3;
+    ctx->stats.mvps += ncols;
   } else if (op == 0) {
     ctx->stats.kernel_launches += apply_A(ctx, X, ldx, Y, ldy, ncols, nullptr);
     ctx->stats.mvps += ncols;
   } else {
     // D and D^H by themselves form right-hand sides of the seed system (b = D^H eta): as apply_seed
-    if (fix_seed(ctx)) {
+    if (fixed) {
       launch_fix_spinors(ctx->wfix, (const double2 *)X, ldx, ctx->F, ctx->ldv, ctx->Fe, ncols, nullptr, ctx->cs);
       launch_dslash_fix(ctx->wfix, op == 1 ? +1 : -1, ctx->F, ctx->Fe, ctx->ldv, nullptr, nullptr, (double2 *)Y, ldy,
                         ncols, nullptr, ctx->cs);

@@ -227,6 +227,9 @@ struct WilsonFix {
 void launch_fix_links(const WilsonFix &op, cudaStream_t s);   // fills flinks and fexp from links
 void launch_fix_spinors(const WilsonFix &op, const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e,
                         int ncols, const int32_t *col_active, cudaStream_t s);
+// both in one launch
+void launch_fix_both(const WilsonFix &op, const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e, int ncols,
+                     cudaStream_t s);
 // few enough tiles x columns for the form with one warp per direction and half-spinor component
 bool fix_few(int64_t sites, int ncols);
 // (q, e) -> (qout, eout), or -> out (doubles, site-major, ldo) when qout is NULL; dot: with D^H only

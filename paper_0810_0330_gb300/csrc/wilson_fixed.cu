@@ -31,33 +31,28 @@ constexpr int kFixPitch = 25;                   // doubles per site of a staged 
 // so the caller's link array may change between calls.  Bound by memory
 // (292 bytes per link).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_fix_links(WilsonFix op, int4 *__restrict__ fl, int32_t *__restrict__ fe) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 4 * op.sites) return;
-  const int64_t mu = idx / op.sites, s = idx - mu * op.sites;
-  double2 u[9];
+
+// One link: limbs and exponent (kExpRaw, kExpZero: zero limbs).  minus_t: the antiperiodic sign.
+SEED_DEV int fix_link(const double2 (&u)[9], double kappa, bool minus_t, int4 (&L)[9]) {
   int bmax = 0;
   bool any = false;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    u[k] = __ldg(op.links + idx * 9 + k);
     bmax = max(bmax, max(fix_bexp(u[k].x), fix_bexp(u[k].y)));
     any |= u[k].x != 0.0 || u[k].y != 0.0;
   }
-  int4 *L = fl + fix_link_at(op, (int)mu, s);
-  const unsigned kh = (unsigned)__double2hiint(op.kappa);
+  const unsigned kh = (unsigned)__double2hiint(kappa);
   const int kb = (int)((kh >> 20) & 0x7ffu);
   const int em = bmax - 1022, ek = kb - 1022;   // |entry| < 2^em, |kappa| < 2^ek
   int g = kExpZero;
   if (bmax == 2047) g = kExpRaw;
-  else if (any && op.kappa != 0.0) g = (em < -kExpLink + 4 || em > kExpLink - 4 || ek < -kExpLink + 4 ||
-                                        ek > kExpLink - 4 || em + ek < -kExpLink + 4 || em + ek > kExpLink - 4)
-                                           ? kExpRaw : em + ek;
+  else if (any && kappa != 0.0) g = (em < -kExpLink + 4 || em > kExpLink - 4 || ek < -kExpLink + 4 ||
+                                     ek > kExpLink - 4 || em + ek < -kExpLink + 4 || em + ek > kExpLink - 4)
+                                        ? kExpRaw : em + ek;
   if (g == kExpRaw || g == kExpZero) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) L[32 * k] = make_int4(0, 0, 0, 0);
-    fe[idx] = g;
-    return;
+    for (int k = 0; k < 9; ++k) L[k] = make_int4(0, 0, 0, 0);
+    return g;
   }
   // upper bound of the row and column sums of |Re| + |Im|, in units of 2^(em - 21)
   unsigned row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
@@ -78,10 +73,9 @@ __global__ void __launch_bounds__(128) k_fix_links(WilsonFix op, int4 *__restric
   for (int a = 0; a < 3; ++a) l1 = max(l1, max(row[a], col[a]));
   const int slack = max(0, 32 - __clz(l1) - 21);   // l1 < 2^(21 + slack)
   g += slack;
-  const bool flip = !((int)kh < 0) ^
-                    (mu == 3 && op.bc_t && s / ((int64_t)op.dims[0] * op.dims[1] * op.dims[2]) == op.dims[3] - 1);
+  const bool flip = !((int)kh < 0) ^ minus_t;
   const unsigned long long km = ((unsigned long long)((kh & 0xfffffu) | 0x100000u) << 32 |
-                                 (unsigned)__double2loint(op.kappa)) << 11;   // kappa 2^(64 - ek)
+                                 (unsigned)__double2loint(kappa)) << 11;   // kappa 2^(64 - ek)
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     int2 l[2];
@@ -96,9 +90,27 @@ __global__ void __launch_bounds__(128) k_fix_links(WilsonFix op, int4 *__restric
       const unsigned long long y = sh > 63 ? 0ull : ((__umul64hi(m, km) >> (sh - 1)) + 1ull) >> 1;
       l[ri] = fix_limbs(y, ((int)hw < 0) ^ flip);
     }
-    L[32 * k] = make_int4(l[0].x, l[0].y, l[1].x, l[1].y);
+    L[k] = make_int4(l[0].x, l[0].y, l[1].x, l[1].y);
   }
-  fe[idx] = g;
+  return g;
+}
+// Link idx = mu * sites + s
+SEED_DEV void fix_link_of(const WilsonFix &op, int4 *fl, int32_t *fe, int64_t idx) {
+  if (idx >= 4 * op.sites) return;
+  const int64_t mu = idx / op.sites, s = idx - mu * op.sites;
+  const bool minus_t = mu == 3 && op.bc_t && s / ((int64_t)op.dims[0] * op.dims[1] * op.dims[2]) == op.dims[3] - 1;
+  double2 u[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) u[k] = __ldg(op.links + idx * 9 + k);
+  int4 l[9];
+  fe[idx] = fix_link(u, op.kappa, minus_t, l);
+  int4 *L = fl + fix_link_at(op, (int)mu, s);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) L[32 * k] = l[k];
+}
+
+__global__ void __launch_bounds__(128) k_fix_links(WilsonFix op, int4 *__restrict__ fl, int32_t *__restrict__ fe) {
+  fix_link_of(op, fl, fe, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 void launch_fix_links(const WilsonFix &op, cudaStream_t s) {
@@ -181,13 +193,9 @@ SEED_DEV int4 fix_out(long long re, long long im, int E, int sh, bool raw, bool 
 }
 
 // grid: tiles * ncols blocks, the column fastest
-__global__ void __launch_bounds__(CT) k_fix_spinors(const double2 *__restrict__ X, int64_t ldx, int4 *__restrict__ q,
-                                                    int64_t ldq, int32_t *__restrict__ e, int64_t sites, int ncols,
-                                                    const int32_t *__restrict__ col_active) {
+SEED_DEV void fix_spinor_tile(const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e, int64_t sites,
+                              int64_t tile, int col) {
   __shared__ double st[32 * kFixPitch];
-  const int64_t tile = blockIdx.x / ncols;
-  const int col = (int)(blockIdx.x - tile * ncols);
-  if (col_active != nullptr && col_active[col] == 0) return;
   const double2 *x = X + (int64_t)col * ldx + tile * 384;
   const int64_t left = 12 * sites - tile * 384;
 #pragma unroll
@@ -199,6 +207,35 @@ __global__ void __launch_bounds__(CT) k_fix_spinors(const double2 *__restrict__ 
   }
   __syncthreads();
   fix_store_tile(st, q + (int64_t)col * ldq + tile * 384, e + (int64_t)col * (ldq / 12) + tile * 32);
+}
+
+__global__ void __launch_bounds__(CT) k_fix_spinors(const double2 *__restrict__ X, int64_t ldx, int4 *__restrict__ q,
+                                                    int64_t ldq, int32_t *__restrict__ e, int64_t sites, int ncols,
+                                                    const int32_t *__restrict__ col_active) {
+  const int64_t tile = blockIdx.x / ncols;
+  const int col = (int)(blockIdx.x - tile * ncols);
+  if (col_active != nullptr && col_active[col] == 0) return;
+  fix_spinor_tile(X, ldx, q, ldq, e, sites, tile, col);
+}
+
+// Links and spinors in one launch, for the smallest operands: the first link_blocks blocks
+// convert CT links each, the others a tile of a column each.
+__global__ void __launch_bounds__(CT) k_fix_both(WilsonFix op, int4 *__restrict__ fl, int32_t *__restrict__ fe,
+                                                 const double2 *__restrict__ X, int64_t ldx, int4 *__restrict__ q,
+                                                 int64_t ldq, int32_t *__restrict__ e, int ncols, unsigned link_blocks) {
+  if (blockIdx.x < link_blocks) {
+    fix_link_of(op, fl, fe, (int64_t)blockIdx.x * CT + threadIdx.x);
+    return;
+  }
+  const int64_t b = blockIdx.x - link_blocks, tile = b / ncols;
+  fix_spinor_tile(X, ldx, q, ldq, e, op.sites, tile, (int)(b - tile * ncols));
+}
+
+void launch_fix_both(const WilsonFix &op, const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e, int ncols,
+                     cudaStream_t s) {
+  const unsigned links = (unsigned)((4 * op.sites + CT - 1) / CT);
+  k_fix_both<<<links + (unsigned)((op.sites + 31) / 32 * ncols), CT, 0, s>>>(
+      op, const_cast<int4 *>(op.flinks), const_cast<int32_t *>(op.fexp), X, ldx, q, ldq, e, ncols, links);
 }
 
 void launch_fix_spinors(const WilsonFix &op, const double2 *X, int64_t ldx, int4 *q, int64_t ldq, int32_t *e,
@@ -360,6 +397,43 @@ SEED_DEV void fix_pair_dir(const WilsonFix &op, const int4 *in, int64_t s, int n
   }
 }
 
+// Component c of spin w of a site: the four directions' partial sums and its own block's value.
+SEED_DEV void fix_spin_sum(const long long (*sacc)[2][12][32], int w, int c, int lane, int4 p, int shs, long long &re,
+                           long long &im) {
+  const int kxy = w < 2 ? w : 3 - w, kzt = w < 2 ? w : w - 2, k = (w < 2 ? 0 : 6) + 2 * c;
+  const long long r = ((long long)p.x << kLimb) + p.y, i = ((long long)p.z << kLimb) + p.w;
+  re = ((r << 1) >> shs) + ((sacc[0][kxy][k][lane] + sacc[1][kxy][k][lane]) + (sacc[2][kzt][k][lane] + sacc[3][kzt][k][lane]));
+  im = ((i << 1) >> shs) + ((sacc[0][kxy][k + 1][lane] + sacc[1][kxy][k + 1][lane]) +
+                            (sacc[2][kzt][k + 1][lane] + sacc[3][kzt][k + 1][lane]));
+}
+
+// The block's result from the sums of warps 0..3 (spin w in v), normalised over the four spins;
+// sites in FP64 (slow) have their 24 reals in sacc.  Contains a CTA barrier.
+SEED_DEV void fix_store_dir(const long long (*sacc)[2][12][32], unsigned (*sO)[2][32], int w, int lane, bool live,
+                            bool slow, int E, const long long (&v)[6], int4 *q, int32_t *e) {
+  if (w < 4) {
+    unsigned mh = 0, ml = 0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) fix_or(v[c], mh, ml);
+    sO[w][0][lane] = mh;
+    sO[w][1][lane] = ml;
+  }
+  __syncthreads();
+  if (!live || w >= 4) return;
+  if (slow) {
+    const double *x = reinterpret_cast<const double *>(&sacc[0][0][0][0]);
+    if (w < 2) fix_store_block([&](int k) { return x[32 * k + lane]; }, w, q + 96 * w, e);
+    return;
+  }
+  const unsigned mh = (sO[0][0][lane] | sO[1][0][lane]) | (sO[2][0][lane] | sO[3][0][lane]);
+  const unsigned ml = (sO[0][1][lane] | sO[1][1][lane]) | (sO[2][1][lane] | sO[3][1][lane]);
+  const int bits = fix_bits(mh, ml), ex = E - 58 + bits, sh = 63 - bits;
+  const bool zero = bits == 0, raw = !zero && (ex < -kExpSite || ex > kExpSite);
+  if (w == 0) *e = zero ? kExpZero : raw ? kExpRaw : ex;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) q[32 * (3 * w + c)] = fix_out(v[2 * c], v[2 * c + 1], E, sh, raw, zero);
+}
+
 template <int S, int OUT>
 __global__ void __launch_bounds__(DT, 3) k_dslash_fix_dir(WilsonFix op, const int4 *__restrict__ in,
                                                           const int32_t *__restrict__ ein, int64_t ldq,
@@ -416,43 +490,14 @@ __global__ void __launch_bounds__(DT, 3) k_dslash_fix_dir(WilsonFix op, const in
   long long v[6];
   if (w < 4) {
     const int shs = min(E - es, 63);
-    const int kxy = w < 2 ? w : 3 - w, kzt = w < 2 ? w : w - 2, r = w < 2 ? 0 : 6;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int4 p = live ? __ldg(in + fix_at(s) + 32 * (3 * w + c)) : make_int4(0, 0, 0, 0);
-#pragma unroll
-      for (int ri = 0; ri < 2; ++ri) {
-        const int k = r + 2 * c + ri;
-        const long long own = ((long long)(ri ? p.z : p.x) << kLimb) + (ri ? p.w : p.y);
-        v[2 * c + ri] = ((own << 1) >> shs) + ((sacc[0][kxy][k][lane] + sacc[1][kxy][k][lane]) +
-                                               (sacc[2][kzt][k][lane] + sacc[3][kzt][k][lane]));
-      }
-    }
-  }
-  if constexpr (OUT == 0) {
-    if (w < 4) {
-      unsigned mh = 0, ml = 0;
-#pragma unroll
-      for (int c = 0; c < 6; ++c) fix_or(v[c], mh, ml);
-      sO[w][0][lane] = mh;
-      sO[w][1][lane] = ml;
-    }
-    __syncthreads();
-    if (!live || w >= 4) return;
-    int4 *q = qout + (int64_t)col * ldq + tile * 384 + lane;
-    int32_t *e = eout + (int64_t)col * (ldq / 12) + s;
-    if (slow) {
-      if (w < 2) fix_store_block([&](int k) { return sslow[k][lane]; }, w, q + 96 * w, e);
-      return;
-    }
-    const unsigned mh = (sO[0][0][lane] | sO[1][0][lane]) | (sO[2][0][lane] | sO[3][0][lane]);
-    const unsigned ml = (sO[0][1][lane] | sO[1][1][lane]) | (sO[2][1][lane] | sO[3][1][lane]);
-    const int bits = fix_bits(mh, ml), ex = E - 58 + bits, sh = 63 - bits;
-    const bool zero = bits == 0, raw = !zero && (ex < -kExpSite || ex > kExpSite);
-    if (w == 0) *e = zero ? kExpZero : raw ? kExpRaw : ex;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      q[32 * (3 * w + c)] = fix_out(v[2 * c], v[2 * c + 1], E, sh, raw, zero);
+      fix_spin_sum(sacc, w, c, lane, live ? __ldg(in + fix_at(s) + 32 * (3 * w + c)) : make_int4(0, 0, 0, 0), shs,
+                   v[2 * c], v[2 * c + 1]);
+  }
+  if constexpr (OUT == 0) {
+    fix_store_dir(sacc, sO, w, lane, live, slow, E, v, qout + (int64_t)col * ldq + tile * 384 + lane,
+                  eout + (int64_t)col * (ldq / 12) + s);
   } else {
     double d[6];
     if (w < 4) {

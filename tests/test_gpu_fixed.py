@@ -125,6 +125,17 @@ def test_fixed_point_operator(seedlib, dims, cols, kind, lk, kappa):
             assert np.all(err <= tol), (bc_t, j, float((err / tol).max()))
 
 
+# tiles x columns up to 152, links and spinors converted in one launch: half a tile, a partial last one, several columns
+@pytest.mark.parametrize("dims,cols", [((2, 2, 2, 2), 1), ((4, 4, 4, 4), 1), ((5, 3, 4, 7), 3), ((2, 3, 2, 5), 2)])
+@pytest.mark.parametrize("kind,lk,kappa", [("gauss", "su3", 0.155), ("site_scales", "su3", -0.4),
+                                           ("component_scales", "su3", 0.155), ("point", "unit", 0.125),
+                                           ("sparse", "some_zero", 0.2), ("gauss", "general", 3e-4),
+                                           ("gauss", "su3", 0.0), ("extreme", "su3", 0.155),
+                                           ("gauss", "extreme", 0.155)])
+def test_fixed_point_operator_few_sites(seedlib, dims, cols, kind, lk, kappa):
+    test_fixed_point_operator(seedlib, dims, cols, kind, lk, kappa)
+
+
 @pytest.mark.parametrize("dims,cols", [((4, 4, 4, 4), 20), ((6, 4, 5, 4), 12)])
 def test_no_less_precise_than_fp64(seedlib, dims, cols):
     """D^H D on random spinors: error against extended precision no larger than the FP64 kernel's."""
