@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from paper_0810_0330_gb300 import inputs as I
-from test_gpu_parity import REL_X, compare_full, csr_ctx, run_gpu, self_sensitivity
+from test_gpu_parity import REL_X, compare_full, csr_ctx, dev_cols, host_cols, run_gpu, self_sensitivity
 
 pytestmark = pytest.mark.gpu
 
@@ -42,4 +42,22 @@ def test_reorth_run_shapes(seedlib, orc, matrix, freq, passes, nrhs):
     m = info1[0]["iters"]
     V = seedlib.seed_get_basis(ctx, m)
     assert np.abs(V.T @ V - np.eye(m)).max() < 1e-12
+    seedlib.seed_destroy(ctx)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [127, 512, 513, 2049, 40001])
+def test_lockstep_cg_kernels_ragged(seedlib, n, precision):
+    """Lockstep CG as step kernels (several elements ahead per thread): lengths at the edges of
+    a thread's four elements and a block's 512.  The claim checked is CG's own: every true
+    residual, recomputed here in FP64 (its rounding is below 1e-14), meets the tolerance."""
+    import scipy.sparse as sp
+    rp, ci, v = band_csr(n, 3)
+    A = sp.csr_matrix((v, ci, rp), shape=(n, n))
+    B = I.gaussian_rhs(n, 3, seed=n)
+    ctx = csr_ctx(seedlib, rp, ci, v, tol_seed=1e-10, tol_rest=1e-10, m_max=50, kernel_path=1, precision=precision)
+    X = dev_cols(np.zeros_like(B))
+    info = seedlib.seed_solve_cg(ctx, dev_cols(B), X)
+    r = np.linalg.norm(B - A @ host_cols(X).real, axis=0) / np.linalg.norm(B, axis=0)
+    assert all(i["converged"] for i in info) and np.all(r <= 1.01e-10), r
     seedlib.seed_destroy(ctx)
