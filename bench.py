@@ -481,9 +481,9 @@ def time_steps(S, torch, p, flush, steps, warmup, clk=None):
 
 
 def dslash_roofline(S, ctx, vol, mixed, dims, ncols_total):
-    """The dominant kernel, the Wilson hopping kernel, timed live on the
-    library's stream: one launch over all CG columns, and the launch shapes the
-    CG graphs issue (one per concurrent column branch)."""
+    """The Wilson hopping kernel timed live on the library's stream: one launch
+    over all CG columns, and the shapes the CG graphs issue (one per concurrent
+    column branch; in FP64 those run in fixed-point integer arithmetic)."""
     shapes = cg_branch_cols(ncols_total)
     if not mixed:
         k_ms = S.seed_time_operator(ctx, 1, ncols_total, 200)
@@ -493,20 +493,21 @@ def dslash_roofline(S, ctx, vol, mixed, dims, ncols_total):
         probe = S.seed_time_fma(S.SEED_F64)["tflops"]
         shape_t = {}
         for c in sorted(set(shapes)):
-            m = S.seed_time_operator(ctx, 1, c, 200)
-            a = FLOPS_PER_SITE_D * vol * c / (m * 1e-3) / 1e12
-            shape_t[str(c)] = {"ms_per_launch": round(m, 5), "achieved": round(a, 4), "frac": round(a / peak, 4)}
+            m = S.seed_time_operator(ctx, 0, c, 200)
+            a = 2 * FLOPS_PER_SITE_D * vol * c / (m * 1e-3) / 1e12
+            shape_t[str(c)] = {"ms_per_apply": round(m, 5), "fp64_equivalent_tflops": round(a, 4)}
         return {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak, 4), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4),
                 "traffic": dslash_traffic() if tuple(dims) == WL["dims"] and ncols_total == 11 else None,
-                "kernel": "k_dslash<+1> (Wilson D, FP64 complex), %d columns in one launch: the work of one CG "
-                          "half-iteration" % ncols_total,
+                "kernel": "k_dslash<+1> (Wilson D in FP64 instructions, the form of a small lattice's seed steps), "
+                          "%d columns in one launch" % ncols_total,
                 "ms_per_launch": round(k_ms, 5), "flops_per_launch": flops,
                 "flops_per_site": FLOPS_PER_SITE_D,
                 "epilogue_flops_per_site": FLOPS_PER_SITE_D_EPILOGUE,
                 "frac_with_epilogue": round((FLOPS_PER_SITE_D + FLOPS_PER_SITE_D_EPILOGUE) * vol * ncols_total /
                                             (k_ms * 1e-3) / 1e12 / peak, 4),
-                "launch_shapes": {"cg_branches": shapes, "per_shape": shape_t},
+                "launch_shapes": {"operator": "D^H D as the CG runs it (k_dslash_fix: integer arithmetic, conversion of "
+                                              "its input included)", "cg_branches": shapes, "per_shape": shape_t},
                 "peak_note": "FP64 pipe from unit counts: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz",
                 "fp64_instructions_per_site": FP64_INSTR_PER_SITE_D,
                 "instruction_mix_ceiling": round(FLOPS_PER_SITE_D / (2.0 * FP64_INSTR_PER_SITE_D), 4),

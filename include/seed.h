@@ -295,8 +295,8 @@ seed_status seed_grad_kappa(seed_ctx *ctx, const void *Lambda, int64_t ldl, cons
  * of seed_time_operator: component k = 3*spin + colour of site s at complex
  * index ((s / 32) * 12 + k) * 32 + s % 32 of a column of length
  * 384 * ceil(sites / 32) (ldx, ldy >= that length); the padding sites of the
- * last tile are written as zeros.  X and Y must not overlap.  Not
- * synchronising. */
+ * last tile are written as zeros.  X and Y must not overlap.  Runs on the
+ * context's stream; not synchronising. */
 seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, void *Y, int64_t ldy,
                        int32_t ncols);
 
@@ -369,7 +369,8 @@ seed_status seed_batch_solve(seed_ctx *const *ctxs, const void *const *B, const 
  * ncols library-owned columns (filled with the byte 0x3F, i.e. normal
  * doubles near 4.8e-4), with CUDA events on that stream
  * around the launches; *ms_per_apply receives the mean device time of one
- * application.  Synchronises.  reps in [1, 100000], ncols in [1, 64]. */
+ * application (Wilson in FP64: op 0 in fixed-point arithmetic above one tile
+ * and column per SM, ops 1 and 2 in FP64 instructions).  Synchronises.  reps in [1, 100000], ncols in [1, 64]. */
 seed_status seed_time_operator(seed_ctx *ctx, int32_t op, int32_t ncols, int32_t reps, double *ms_per_apply);
 
 /* Measurement helper (no counterpart in the paper): the FMA rate of the FP64
