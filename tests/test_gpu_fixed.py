@@ -280,3 +280,23 @@ def test_apply_on_the_callers_stream(seedlib):
             X.zero_()
             assert np.array_equal(Y.cpu().numpy(), ref)
     seedlib.seed_destroy(ctx)
+
+
+@pytest.mark.parametrize("nrhs", [2, 3, 4, 5, 8])
+def test_seeding_products_of_any_width(seedlib, orc, nrhs):
+    """The block flush with 1, 2, 3, 4 and 4 + 3 seeded systems against the oracle; bounds as in
+    the parity tests (the oracle's own sensitivity to a last-bit change)."""
+    from paper_0810_0330_gb300 import inputs as I
+    from test_gpu_parity import REL_X, compare_full, run_gpu, self_sensitivity, wilson_ctx
+    dims, kappa = (3, 3, 5, 5), 0.13
+    U = I.random_su3_links(dims, 0.3, seed=4)
+    B = I.gaussian_rhs(12 * 225, nrhs, seed=5, complex_=True)
+    kw = dict(m_max=300, reorth_freq=9)
+    ctx = wilson_ctx(seedlib, dims, kappa, U, tol_seed=1e-10, tol_rest=1e-8, **kw)
+    info1, info2, Xs, X = run_gpu(seedlib, ctx, B)
+    op = orc.Operator.wilson(dims, kappa, U)
+    ref = orc.seed_solve_all(op, B, tol_seed=1e-10, tol_rest=1e-8, **kw)
+    s_seed, s_final = self_sensitivity(orc, op, B, ref, cols=(1,), tol=1e-10, **kw)
+    compare_full(ref, info1, info2, Xs, X, "wilson-flush", seeded_tol=max(REL_X, 10 * s_seed),
+                 final_tol=max(REL_X, 10 * s_final))
+    seedlib.seed_destroy(ctx)
