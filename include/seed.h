@@ -296,7 +296,12 @@ seed_status seed_grad_kappa(seed_ctx *ctx, const void *Lambda, int64_t ldl, cons
  * index ((s / 32) * 12 + k) * 32 + s % 32 of a column of length
  * 384 * ceil(sites / 32) (ldx, ldy >= that length); the padding sites of the
  * last tile are written as zeros.  X and Y must not overlap.  Runs on the
- * context's stream; not synchronising. */
+ * context's stream; not synchronising.
+ *   In a stream capture: the call needs room for ncols columns from an earlier
+ * call; the graph is valid until seed_destroy.  Graphs of ops 1, 2, 4, 5, 6 and 7 (and of
+ * ops 0 and 3 on a CSR context) use nothing but the operator, X and Y.  Graphs of ops 0 and 3 on a
+ * Wilson context use the context's work space as well: a replay must not overlap in
+ * time with other calls on the context or with another such replay. */
 seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, void *Y, int64_t ldy,
                        int32_t ncols);
 

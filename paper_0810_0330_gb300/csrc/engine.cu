@@ -94,6 +94,8 @@ struct seed_ctx {
   // multi-column work space (grown on demand): R0 / R, P, Q, Wilson temp
   int cap_cols = 0;
   void *R = nullptr, *P = nullptr, *Q = nullptr, *T = nullptr;
+  bool captured = false;               // a caller's graph names work space of seed_apply (T, F, Fe, P32, T32)
+  std::vector<void *> kept;            // such work space after growth: lives as long as the context
 
   // lockstep CG
   double *cg_d = nullptr;     // 5 * kMaxRhs doubles
@@ -306,13 +308,17 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
   if (cols <= ctx->cap_cols) return SEED_OK;
   cudaStreamSynchronize(ctx->cs);
   cudaEventSynchronize(ctx->ev_apply);
-  cudaFree(ctx->R); cudaFree(ctx->P); cudaFree(ctx->Q); cudaFree(ctx->T); cudaFree(ctx->F); cudaFree(ctx->Fe);
-  cudaFree(ctx->dotpart);
+  for (void *q : {ctx->T, (void *)ctx->F, (void *)ctx->Fe, ctx->P32, ctx->T32}) {
+    if (ctx->captured && q) ctx->kept.push_back(q);   // a replay may still come
+    else cudaFree(q);
+  }
+  ctx->captured = false;
+  cudaFree(ctx->R); cudaFree(ctx->P); cudaFree(ctx->Q); cudaFree(ctx->dotpart);
   ctx->R = ctx->P = ctx->Q = ctx->T = nullptr;
   ctx->F = nullptr;
   ctx->Fe = nullptr;
   ctx->dotpart = nullptr;
-  cudaFree(ctx->R32); cudaFree(ctx->P32); cudaFree(ctx->Q32); cudaFree(ctx->T32); cudaFree(ctx->E32);
+  cudaFree(ctx->R32); cudaFree(ctx->Q32); cudaFree(ctx->E32);
   ctx->R32 = ctx->P32 = ctx->Q32 = ctx->T32 = ctx->E32 = nullptr;
   ctx->cap_cols = 0;
   // graphs captured with the old buffers are stale
@@ -413,8 +419,11 @@ int apply_seed(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, 
 
 // Y = op X with the FP32 copy of the operator (mixed precision), op 0 = A, 1 = D, 2 = D^H.
 // tiled: X and Y in the solver's tiled FP32 layout (else the caller's site-major one; on large
-// lattices that goes through tiled columns in P32 and T32).  Returns the kernel count.
-int apply_32(seed_ctx *ctx, int op, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, bool tiled) {
+// lattices that goes through tiled columns in P32 and T32, or without work space for D and D^H
+// where the call is captured: a replay may run beside the context's other work).  Returns the
+// kernel count.
+int apply_32(seed_ctx *ctx, int op, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, bool tiled,
+             bool capturing = false) {
   if (ctx->kind == 0) {
     launch_csr_spmv32(ctx->csr32, (const float *)X, ldx, (float *)Y, ldy, ncols, nullptr, ctx->cs);
     return 1;
@@ -424,14 +433,18 @@ int apply_32(seed_ctx *ctx, int op, const void *X, int64_t ldx, void *Y, int64_t
   float2 *y = (float2 *)Y, *t = (float2 *)ctx->T32;
   const int64_t ld = ctx->ldv;
   if (!tiled && dslash32_tiles(w.sites)) {
+    if (op != 0 && capturing) {
+      launch_wilson_dslash32_user(w, op == 1 ? +1 : -1, x, ldx, false, y, ldy, ncols, ctx->cs);
+      return 1;
+    }
     float2 *p = (float2 *)ctx->P32;
     launch_tile32(x, ldx, p, ld, w.sites, ncols, ctx->cs);
     if (op != 0) {
-      launch_wilson_dslash32_user(w, op == 1 ? +1 : -1, p, ld, y, ldy, ncols, ctx->cs);
+      launch_wilson_dslash32_user(w, op == 1 ? +1 : -1, p, ld, true, y, ldy, ncols, ctx->cs);
       return 2;
     }
     launch_wilson_dslash32(w, +1, p, ld, t, ld, ncols, nullptr, true, ctx->cs);
-    launch_wilson_dslash32_user(w, -1, t, ld, y, ldy, ncols, ctx->cs);
+    launch_wilson_dslash32_user(w, -1, t, ld, true, y, ldy, ncols, ctx->cs);
     return 3;
   }
   if (op != 0) {
@@ -1681,17 +1694,20 @@ struct StreamScope {
 // The operator by itself runs on the caller's stream, without the two event waits of StreamScope (D^H D
 // on 2048^2 CSR rows 60.6 -> 59.4 us a call).  Every other call starts
 // behind that stream; what frees work space without starting there waits for ev_apply.
+// Under a capture nothing is recorded for replays to come: work space that the graph
+// names is kept until seed_destroy (ensure_cols).
 struct ApplyScope {
   seed_ctx *ctx;
   cudaStream_t own;
+  bool capturing;
   explicit ApplyScope(seed_ctx *c) : ctx(c), own(c->cs) {
     ctx->links_ready = false;   // ensure_fixed
     ctx->cs = ctx->user_stream;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    capturing = cudaStreamIsCapturing(ctx->cs, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
   }
   ~ApplyScope() {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->cs, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone)
-      cudaEventRecord(ctx->ev_apply, ctx->cs);
+    if (!capturing) cudaEventRecord(ctx->ev_apply, ctx->cs);
     ctx->cs = own;
   }
 };
@@ -1738,6 +1754,7 @@ void destroy(seed_ctx *ctx) {
                   ctx->tc_err, ctx->rhpart, ctx->Hrows};
   for (void *q : ptrs)
     if (q) cudaFree(q);
+  for (void *q : ctx->kept) cudaFree(q);
   if (ctx->h_flags) cudaFreeHost(ctx->h_flags);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
   if (ctx->h_gerr) cudaFreeHost(ctx->h_gerr);
@@ -2090,11 +2107,14 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   TRY(ensure_cols(ctx, ncols));
   ApplyScope scope(ctx);
   const bool few = op == 0 && ctx->kind == 1 && !fix_pays(ctx, ncols);   // links and spinors converted in one launch
-  const bool fixed = ctx->kind == 1 && (op == 0 || (op < 3 && fix_seed(ctx))) && try_fixed(ctx, !few);
+  // D and D^H in a capture take no work space: their graphs depend on the operator, X and Y alone
+  const bool fixed = ctx->kind == 1 && (op == 0 || (op < 3 && fix_seed(ctx) && !scope.capturing)) && try_fixed(ctx, !few);
+  if (scope.capturing && ctx->kind == 1 && (op == 0 || op == 3)) ctx->captured = true;
   if (op == 3) {
     ctx->stats.kernel_launches += apply_32(ctx, 0, X, ldx, Y, ldy, ncols, false);
   } else if (op >= 4) {
-    ctx->stats.kernel_launches += apply_32(ctx, (op == 4 || op == 6) ? 1 : 2, X, ldx, Y, ldy, ncols, tiled);
+    ctx->stats.kernel_launches +=
+        apply_32(ctx, (op == 4 || op == 6) ? 1 : 2, X, ldx, Y, ldy, ncols, tiled, scope.capturing);
   } else if (few && fixed) {   // 4^4, one column: 24.6 -> 18.5 us a call (two FP64 launches before)
     launch_fix_both(ctx->wfix, (const double2 *)X, ldx, ctx->F, ctx->ldv, ctx->Fe, ncols, ctx->cs);
     launch_dslash_fix(ctx->wfix, +1, ctx->F, ctx->Fe, ctx->ldv, fix_T(ctx), fix_Te(ctx), nullptr, 0, ncols, nullptr,

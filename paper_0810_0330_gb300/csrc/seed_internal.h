@@ -204,10 +204,10 @@ void launch_wilson_dslash32(const WilsonOp32 &op, int sign, const float2 *in, in
                             int ncols, const int32_t *col_active, bool tiled, cudaStream_t s,
                             const CgDot<float2> *dot = nullptr);   // dot: tiled only
 // The caller's layout at sizes where dslash32_tiles: its columns into the tiled layout, and the
-// operator from there into the caller's layout
+// operator into the caller's layout, from there or (tiled = false) from the caller's layout
 bool dslash32_tiles(int64_t sites);
 void launch_tile32(const float2 *in, int64_t ldi, float2 *out, int64_t ldo, int64_t sites, int ncols, cudaStream_t s);
-void launch_wilson_dslash32_user(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, float2 *out,
+void launch_wilson_dslash32_user(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, bool tiled, float2 *out,
                                  int64_t ldo, int ncols, cudaStream_t s);
 void launch_links_soa32(const double2 *links, float2 *out, int64_t sites, cudaStream_t s);
 

@@ -35,19 +35,19 @@ SEED_DEV V ldro(const V *p) {
   else return __ldg(p);
 }
 
-template <bool VEC>
+template <bool VEC, bool L2ONLY = false>
 SEED_DEV void load_spinor(const float2 *__restrict__ p, float2 (&ps)[12]) {
   if constexpr (VEC) {
     const float4 *q = reinterpret_cast<const float4 *>(p);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const float4 v = __ldg(q + k);
+      const float4 v = ldro<L2ONLY>(q + k);
       ps[2 * k] = make_float2(v.x, v.y);
       ps[2 * k + 1] = make_float2(v.z, v.w);
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) ps[k] = __ldg(p + k);
+    for (int k = 0; k < 12; ++k) ps[k] = ldro<L2ONLY>(p + k);
   }
 }
 
@@ -184,6 +184,14 @@ __global__ void __launch_bounds__(128) k_dslash32(WilsonOp32 op, const float2 *_
 // ---------------------------------------------------------------------------
 constexpr int64_t kSiteKernelSites = 65536;
 
+// Layout of the site kernel's input: the solver's, or the caller's (read as float4 where it is aligned)
+constexpr int kInTiled = 0, kInSites = 1, kInSites4 = 2;
+template <int IN, bool L2ONLY>
+SEED_DEV void load_site(const float2 *__restrict__ in, int64_t q, float2 (&ps)[12]) {
+  if constexpr (IN == kInTiled) load_spinor_tiled<L2ONLY>(in, q, ps);
+  else load_spinor<IN == kInSites4, L2ONLY>(in + 12 * q, ps);
+}
+
 // direction MU of site s for the columns set in jm (bit j: column j of the
 // pair); MU == 0 starts the sums.  Cache policy: the x and y neighbours of a
 // block's sites lie in the block's own or adjacent 32-site tiles, which its
@@ -193,7 +201,7 @@ constexpr int64_t kSiteKernelSites = 65536;
 // on GB300 (11 columns): 16^3 x 32 114.9 -> 103.3 us and 32^3 x 64 1985 ->
 // 1879 us together with the streaming stores of the epilogue; same results
 // bit for bit.
-template <int MU, int S>
+template <int MU, int S, int IN>
 SEED_DEV void site_dir2(const WilsonOp32 &op, const float2 *__restrict__ in, int64_t ldi, int64_t s, int32_t nf,
                         int32_t nb, unsigned negf, unsigned negb, unsigned jm, float2 (&acc)[2][12]) {
   constexpr bool kFar = MU >= 2;
@@ -206,7 +214,7 @@ SEED_DEV void site_dir2(const WilsonOp32 &op, const float2 *__restrict__ in, int
     for (int j = 0; j < 2; ++j) {
       if (jm & (1u << j)) {
         float2 p[12];
-        load_spinor_tiled<kFar>(in + j * ldi, nf, p);
+        load_site<IN, kFar>(in + j * ldi, nf, p);
         hop_r<MU, S, true, MU == 0>(p, u, negf, acc[j]);
       }
     }
@@ -219,7 +227,7 @@ SEED_DEV void site_dir2(const WilsonOp32 &op, const float2 *__restrict__ in, int
     for (int j = 0; j < 2; ++j) {
       if (jm & (1u << j)) {
         float2 p[12];
-        load_spinor_tiled<kFar>(in + j * ldi, nb, p);
+        load_site<IN, kFar>(in + j * ldi, nb, p);
         hop_r<MU, -S, false, false>(p, u, negb, acc[j]);
       }
     }
@@ -228,9 +236,9 @@ SEED_DEV void site_dir2(const WilsonOp32 &op, const float2 *__restrict__ in, int
 
 // Grid: one block per (128 sites, column pair), the pair fastest, so that the
 // pairs of one site block run together and their link loads hit L2.
-// Input in the tiled layout.  USER: the result in the caller's site-major layout, staged
-// through shared memory so that the stores are contiguous.
-template <int S, bool DOT = false, bool USER = false>
+// USER: the result in the caller's site-major layout, staged through shared memory so that
+// the stores are contiguous; there the input may be in that layout too (IN).
+template <int S, bool DOT = false, bool USER = false, int IN = kInTiled>
 __global__ void __launch_bounds__(128, 4) k_dslash32_site(WilsonOp32 op, const float2 *__restrict__ in, int64_t ldi,
                                                           float2 *__restrict__ out, int64_t ldo,
                                                           const int32_t *__restrict__ col_active, int ncols,
@@ -260,14 +268,15 @@ __global__ void __launch_bounds__(128, 4) k_dslash32_site(WilsonOp32 op, const f
       if (t == op.dims[3] - 1) negf = CxBits<float2>::sign;
       if (t == 0) negb = CxBits<float2>::sign;
     }
-    site_dir2<0, S>(op, in, ldi, s, a.x, a.y, 0u, 0u, jm, acc);
-    site_dir2<1, S>(op, in, ldi, s, a.z, a.w, 0u, 0u, jm, acc);
-    site_dir2<2, S>(op, in, ldi, s, b.x, b.y, 0u, 0u, jm, acc);
-    site_dir2<3, S>(op, in, ldi, s, b.z, b.w, negf, negb, jm, acc);
+    site_dir2<0, S, IN>(op, in, ldi, s, a.x, a.y, 0u, 0u, jm, acc);
+    site_dir2<1, S, IN>(op, in, ldi, s, a.z, a.w, 0u, 0u, jm, acc);
+    site_dir2<2, S, IN>(op, in, ldi, s, b.x, b.y, 0u, 0u, jm, acc);
+    site_dir2<3, S, IN>(op, in, ldi, s, b.z, b.w, negf, negb, jm, acc);
   }
   const float mk = (float)(-op.kappa);
-  const int64_t so = (s >> 5) * 384 + (s & 31);
-  constexpr int kStride = 32;
+  static_assert(IN == kInTiled || USER, "tiled results come from tiled columns");
+  const int64_t so = IN == kInTiled ? (s >> 5) * 384 + (s & 31) : 12 * s;
+  constexpr int kStride = IN == kInTiled ? 32 : 1;
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     if (!(jm & (1u << j))) continue;
@@ -361,14 +370,22 @@ void launch_tile32(const float2 *in, int64_t ldi, float2 *out, int64_t ldo, int6
   k_tile32<<<dim3((unsigned)((sites + 31) / 32), (unsigned)ncols), 128, 0, s>>>(in, ldi, out, ldo, sites);
 }
 
-void launch_wilson_dslash32_user(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, float2 *out,
-                                 int64_t ldo, int ncols, cudaStream_t s) {
+template <int IN>
+static void dslash32_user(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, float2 *out, int64_t ldo,
+                          int ncols, cudaStream_t s) {
   const unsigned g = (unsigned)(((op.sites + 127) / 128) * ((ncols + 1) / 2));
   const CgDot<float2> d{};
   if (sign > 0)
-    k_dslash32_site<+1, false, true><<<g, 128, 0, s>>>(op, in, ldi, out, ldo, nullptr, ncols, d);
+    k_dslash32_site<+1, false, true, IN><<<g, 128, 0, s>>>(op, in, ldi, out, ldo, nullptr, ncols, d);
   else
-    k_dslash32_site<-1, false, true><<<g, 128, 0, s>>>(op, in, ldi, out, ldo, nullptr, ncols, d);
+    k_dslash32_site<-1, false, true, IN><<<g, 128, 0, s>>>(op, in, ldi, out, ldo, nullptr, ncols, d);
+}
+
+void launch_wilson_dslash32_user(const WilsonOp32 &op, int sign, const float2 *in, int64_t ldi, bool tiled, float2 *out,
+                                 int64_t ldo, int ncols, cudaStream_t s) {
+  if (tiled) dslash32_user<kInTiled>(op, sign, in, ldi, out, ldo, ncols, s);
+  else if ((uintptr_t)in % 16 == 0 && ldi % 2 == 0) dslash32_user<kInSites4>(op, sign, in, ldi, out, ldo, ncols, s);
+  else dslash32_user<kInSites>(op, sign, in, ldi, out, ldo, ncols, s);
 }
 
 // Column groups: enough blocks to give every SM about four, otherwise all
