@@ -1789,7 +1789,10 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     gather(nullptr, 0, nullptr, r, 2, s_sum);
     hc = passes > 1 ? s_sum[1] : 0.0;
     if (hc != 0.0) f = fma(-hc, v, f);
-    if (scalar) seed_finish<double, false>(bl, fmax(0.0, fma(-hc, hc, s_sum[0])));
+    if (scalar) {
+      const double ff = fma(-hc, hc, s_sum[0]);   // ||f||^2; NaN stays NaN (fmax would drop it)
+      seed_finish<double, false>(bl, ff < 0.0 ? 0.0 : ff);
+    }
     vlast = v;
     par ^= 1;
   }
