@@ -1302,11 +1302,14 @@ __global__ void __launch_bounds__(CRT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> o
 //    of the normalization come with the second pass's products: that pass changes them by
 //    the square of its coefficients, below rounding.  The last projection's
 //    coefficient h and ||f||^2 come together, and f - h v_i is formed by whoever reads f next;
-//  - a block's rows of V stay in shared memory, as 57-bit integers in two limbs
-//    (|V| <= 1), and the products with them are integer multiply-adds
-//    (wilson_fixed.cuh has the rates): per block and column exact sums of products cut off 2^-55
-//    below the block's largest factor, which is below the rounding errors of the
-//    FP64 sums they replace.  Columns past kcap (shared memory) are read from V in FP64.
+//  - a block's rows of V stay in shared memory, as 56-bit integers in two limbs with one
+//    exponent per column, and the products with them are integer multiply-adds
+//    (wilson_fixed.cuh has the rates): factors rounded 2^-57 below the block's largest, the
+//    products of the two low limbs dropped (at most 2^-58 of the largest each, either sign), the
+//    sums exact and rounded once.  Against exact sums of random unit vectors (emulated with
+//    the kernel's shapes): V^H v rms 1.2e-18 at n = 4096, 0.8e-18 at 9216, FP64 sums 3.2e-18
+//    and 2.8e-18; V H of 2 to 300 columns 0.2 to 0.9 of the FP64 sums' error.
+//    Columns past kcap (shared memory) are read from V in FP64.
 //   H = V_{<i}^H [v_i u]: per block and column the sums over the block's rows,
 //   written to hpart[(2 c + v) G + b]; after a barrier block b sums the values [2 k b /
 //   G, 2 k (b + 1) / G) over the blocks in block order into H; after a second
@@ -1323,7 +1326,10 @@ constexpr int kRunRegion = 32;                 // doubles per block in a scalar 
 constexpr int kRunMaxRhs = kReorthRunMaxRhs;   // alpha_i and g^2..g^16 in one region row
 constexpr int RT = 256;                        // threads per block
 constexpr int kRunSmem = 100 * 1024;           // shared memory of V's rows and H: two problems' blocks fit an SM
-constexpr int kVBits = 57, kYBits = 55, kHBits = 51;   // V, the block's v_i / u / f, H: |I| < 2^bits
+// V's rows of a block by column, the block's v_i / u / f, H 2^(its column's exponent): |I| <= 2^kBits.
+// Bounds: |hi| <= 2^28, |lo| <= 2^27, so a sum of up to 64 products has |hi hi| parts below 2^62, cross
+// terms too; 50 or more columns per thread do not fit in shared memory.
+constexpr int kBits = 56;
 
 // after the barrier: S[q] = sum over blocks (in block order) of region[b * kRunRegion + q], q < nv
 SEED_DEV void reduce_region(const double *region, int nv, double *S) {
@@ -1381,33 +1387,46 @@ SEED_DEV void gather(const double *hpart, int k, double *H, const double *region
   __syncthreads();
 }
 
-// x 2^p as a 64-bit integer in two limbs hi 2^28 + lo, both with x's sign; x not finite or
-// zero: 0.  |x| 2^p < 2^57.  (p <= 1200: a subnormal x is cut off to zero.)
+// x 2^p rounded to a 64-bit integer, as two limbs hi 2^28 + lo with |lo| <= 2^27; x not finite or
+// zero: 0.  |x| 2^p <= 2^kBits.  (A subnormal x is cut off to zero.)
 SEED_DEV int2 limbs(double x, int p) {
   const unsigned hw = (unsigned)__double2hiint(x);
   const int be = (int)((hw >> 20) & 0x7ffu), sh = 1075 - be - p;   // mantissa (53 bits) >> sh
   if (be == 0 || be == 2047 || sh > 53) return make_int2(0, 0);
   const unsigned long long m =
       (unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x);
-  const unsigned long long y = sh > 0 ? m >> sh : m << -sh;
-  const int s = (int)hw >> 31, hi = (int)(y >> 28), lo = (int)(y & 0xfffffffu);
-  return make_int2((hi ^ s) - s, (lo ^ s) - s);
+  const long long y = (long long)(sh > 0 ? ((m >> (sh - 1)) + 1) >> 1 : m << -sh);
+  const long long v = (int)hw < 0 ? -y : y;
+  const int hi = (int)((v + (1 << 27)) >> 28);
+  return make_int2(hi, (int)(v - ((long long)hi << 28)));
 }
 // |x| < 2^(the result); a large negative number for zero
 SEED_DEV int exp2_above(double x) {
   const int be = (__double2hiint(x) >> 20) & 0x7ff;
   return be == 0 ? -1100 : be - 1022;
 }
-// (hi 2^56 + mid 2^28) 2^-p as a double
-SEED_DEV double limb_sum(long long hi, long long mid, int p) {
-  return scalbn((double)(hi + (mid >> 28)), 56 - p);
+// hi + mid 2^-28, rounded
+SEED_DEV long long limb_carry(long long hi, long long mid) { return hi + ((mid + (1 << 27)) >> 28); }
+
+// One warp: column c of the block's rows of V into shared memory; lane l has row l's value in x0
+// and row l + 32's in x1 (zero past the block's rows).
+template <int RB>
+SEED_DEV void keep_column(int2 *sV, int *s_ve, int c, double x0, double x1) {
+  const int lane = threadIdx.x & 31;
+  int e = max(exp2_above(x0), exp2_above(x1));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  int2 *col = sV + (int64_t)c * (RB + 1);
+  if (lane < RB) col[lane] = limbs(x0, kBits - e);
+  if (RB > 32) col[32 + lane] = limbs(x1, kBits - e);
+  if (lane == 0) s_ve[c] = e;
 }
 
 // hpart[(2 c + v) G + b] = sum over the block's rows r of V[c][row0 + r] y_v[r], c < k.  s_yl: the
-// limbs of y 2^(kYBits - ye[v]).  Up to four threads share a column's rows while k leaves
+// limbs of y 2^(kBits - ye[v]); ve: V's exponents.  Up to four threads share a column's rows while k leaves
 // threads idle.
 template <int RB>
-SEED_DEV void col_dots(const int2 *sV, int kcap, const double *V, int64_t ldv, int64_t row0, int rows, int k,
+SEED_DEV void col_dots(const int2 *sV, const int *ve, int kcap, const double *V, int64_t ldv, int64_t row0, int rows, int k,
                        const double (*y)[RB], const int4 *s_yl, const int *ye, double *hpart) {
   const int G = gridDim.x;
   const int kf = k < kcap ? k : kcap;
@@ -1437,8 +1456,9 @@ SEED_DEV void col_dots(const int2 *sV, int kcap, const double *V, int64_t ldv, i
       m1 += __shfl_xor_sync(0xffffffffu, m1, o);
     }
     if (c < kf && part == 0) {
-      hpart[(int64_t)(2 * c) * G + blockIdx.x] = limb_sum(a0, m0, kVBits + kYBits - ye[0]);
-      hpart[(int64_t)(2 * c + 1) * G + blockIdx.x] = limb_sum(a1, m1, kVBits + kYBits - ye[1]);
+      const int p = 56 - 2 * kBits + ve[c];
+      hpart[(int64_t)(2 * c) * G + blockIdx.x] = scalbn((double)limb_carry(a0, m0), p + ye[0]);
+      hpart[(int64_t)(2 * c + 1) * G + blockIdx.x] = scalbn((double)limb_carry(a1, m1), p + ye[1]);
     }
   }
   for (int c = kcap + threadIdx.x; c < k; c += RT) {
@@ -1456,19 +1476,19 @@ SEED_DEV void col_dots(const int2 *sV, int kcap, const double *V, int64_t ldv, i
 
 // sub[v][r] = sum over c < k of V[c][row0 + r] H[2 c + v]: thread (r, g) of the
 // block (r = t mod RB, g = t / RB) sums the columns c = g, g + groups, ... of row r, then
-// each output adds its group sums in group order.  H comes from L2 once: as limbs with
-// one exponent per v into s_hl.
+// each output adds its group sums.  H comes from L2 once: times 2^(V's exponent of the column),
+// as limbs with one exponent per v, into s_hl.
 template <int RB>
-SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V, int64_t ldv, int64_t row0, int rows,
+SEED_DEV void rows_times_h(const int2 *sV, const int *ve, int kcap, int4 *s_hl, const double *V, int64_t ldv, int64_t row0, int rows,
                            int k, const double *H, double (*sub)[RB], long long (*sred)[2 * RB], double (*stail)[2 * RB],
                            int (*s_he)[2]) {
   constexpr int kGroups = RT / RB;
   const int kf = k < kcap ? k : kcap;   // columns in shared memory
-  int e0 = -1100, e1 = -1100;
+  int e0 = -3000, e1 = -3000;   // below any sum of two exponents
   for (int c = threadIdx.x; c < kf; c += RT) {
     const double2 h = __ldcg(reinterpret_cast<const double2 *>(H) + c);
-    e0 = max(e0, exp2_above(h.x));
-    e1 = max(e1, exp2_above(h.y));
+    e0 = max(e0, exp2_above(h.x) + ve[c]);
+    e1 = max(e1, exp2_above(h.y) + ve[c]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1487,7 +1507,7 @@ SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V
   }
   for (int c = threadIdx.x; c < kf; c += RT) {
     const double2 h = __ldcg(reinterpret_cast<const double2 *>(H) + c);
-    const int2 p = limbs(h.x, kHBits - e0), q = limbs(h.y, kHBits - e1);
+    const int2 p = limbs(h.x, kBits - e0 + ve[c]), q = limbs(h.y, kBits - e1 + ve[c]);
     s_hl[c] = make_int4(p.x, p.y, q.x, q.y);
   }
   __syncthreads();
@@ -1504,9 +1524,8 @@ SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V
     m1 = (long long)x.x * q.w + m1;
     m1 = (long long)x.y * q.z + m1;
   }
-  // |V H| sums are below 2^(kVBits + kHBits) sqrt(k) in all: the shifted sums add up exactly
-  sred[grp][r] = a0 + (m0 >> 28);
-  sred[grp][RB + r] = a1 + (m1 >> 28);
+  sred[grp][r] = limb_carry(a0, m0);
+  sred[grp][RB + r] = limb_carry(a1, m1);
   const bool tail = k > kf;
   if (tail) {
     double pv = 0.0, pf = 0.0;
@@ -1524,10 +1543,14 @@ SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V
   __syncthreads();
   if ((int)threadIdx.x < 2 * RB) {
     const int q = threadIdx.x;
-    long long t = sred[0][q];
+    long long t = 0;   // the groups' sums in two parts: all of them could pass 63 bits
+    int lo = 0;
 #pragma unroll
-    for (int g2 = 1; g2 < kGroups; ++g2) t += sred[g2][q];
-    double d = limb_sum(t, 0, kVBits + kHBits - (q < RB ? e0 : e1));
+    for (int g2 = 0; g2 < kGroups; ++g2) {
+      t += sred[g2][q] >> 8;
+      lo += (int)(sred[g2][q] & 255);
+    }
+    double d = scalbn(fma((double)t, 256.0, (double)lo), 56 - 2 * kBits + (q < RB ? e0 : e1));
     if (tail)
       for (int g2 = 0; g2 < kGroups; ++g2) d += stail[g2][q];
     sub[q / RB][q % RB] = d;
@@ -1536,7 +1559,7 @@ SEED_DEV void rows_times_h(const int2 *sV, int kcap, int4 *s_hl, const double *V
 }
 
 template <int RB>
-__global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, CsrOp op, double *f2, GridSync g,
+__global__ void __launch_bounds__(RT, 2) k_seed_run_csr_reorth(SeedBufs<double> b, CsrOp op, double *f2, GridSync g,
                                                             double *bpart, double *hpart, double *H, int freq,
                                                             int passes, int i_stop, int kcap) {
   static_assert(2 * RB <= RT && RT % RB == 0, "rows per block");
@@ -1554,6 +1577,7 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
   extern __shared__ int4 s_run[];
   int4 *const s_hl = s_run;                                  // [kcap] limbs of H
   int2 *const sV = reinterpret_cast<int2 *>(s_run + kcap);   // [kcap][RB + 1] limbs of this block's rows of V
+  int *const s_ve = reinterpret_cast<int *>(sV + (int64_t)kcap * (RB + 1));   // [kcap] their exponents by column
   unsigned epoch = 0;
   int par = 0, reg = 0;
   local_load(b, L);
@@ -1610,7 +1634,7 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
         e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
       }
       for (int r = threadIdx.x; r < RB; r += 32) {
-        const int2 p = limbs(s_y[0][r], kYBits - e0), q = limbs(s_y[1][r], kYBits - e1);
+        const int2 p = limbs(s_y[0][r], kBits - e0), q = limbs(s_y[1][r], kBits - e1);
         s_yl[r] = make_int4(p.x, p.y, q.x, q.y);
       }
       if (threadIdx.x == 0) {
@@ -1620,16 +1644,23 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     }
     __syncthreads();
   };
-  // column c of this block's rows of V in shared memory
-  auto keep = [&](int c, double v) {
-    if (c < kcap && (int)threadIdx.x < RB) sV[(int64_t)c * (RB + 1) + threadIdx.x] = limbs(own ? v : 0.0, kVBits);
+  // column c of this block's rows of V, staged in s_y[0] before a CTA barrier, into shared memory:
+  // the fourth warp, beside the first two's row sums
+  auto keep = [&](int c) {
+    if (threadIdx.x >> 5 != 3 || c >= kcap) return;
+    const int lane = threadIdx.x & 31;
+    keep_column<RB>(sV, s_ve, c, lane < RB ? s_y[0][lane] : 0.0, RB > 32 ? s_y[0][(RB > 32 ? 32 : 0) + lane] : 0.0);
   };
   const bool scalar = threadIdx.x == RT - 32;   // runs the recurrence's scalar code beside the others
   double f = own ? b.f[e] : 0.0;   // this row's f, final
   double hc = 0.0;                 // f in global memory is still to have hc v_{i-1} subtracted
   double vlast = 0.0;              // this row's v_{i-1}
   int il = L.st.i - 1;             // last finished step
-  for (int c = 0; c < il; ++c) keep(c, own ? b.V[(int64_t)c * ldv + e] : 0.0);   // (a run that starts later)
+  for (int c = threadIdx.x >> 5; c < min(il, kcap); c += RT / 32) {   // (a run that starts later)
+    const int lane = threadIdx.x & 31;
+    const double *vc = b.V + (int64_t)c * ldv + row0;
+    keep_column<RB>(sV, s_ve, c, lane < min(RB, rows) ? vc[lane] : 0.0, RB > 32 && lane + 32 < rows ? vc[lane + 32] : 0.0);
+  }
   if (il > 0 && own) vlast = b.V[(int64_t)(il - 1) * ldv + e];
   // The LU update's vectors of a step (w_i, x^1 += zeta_i w_i, x^j += eta^j w_i) wait for the next
   // barrier's window: pend, with the step's v_i as it was before its reorthogonalization.
@@ -1699,7 +1730,7 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     double *r = region();
     if (ro) {
       stage_y(v, u);
-      col_dots<RB>(sV, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
+      col_dots<RB>(sV, s_ve, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
     } else {
       __syncthreads();
     }
@@ -1716,10 +1747,13 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     il = i;
     r = region();
     if (!ro) {
-      keep(k, v);
       if (own) fn[e] = f;
-      if ((int)threadIdx.x < RB) s_val[0][threadIdx.x] = own ? f * f : 0.0;
+      if ((int)threadIdx.x < RB) {
+        s_val[0][threadIdx.x] = own ? f * f : 0.0;
+        s_y[0][threadIdx.x] = v;
+      }
       __syncthreads();
+      keep(k);
       row_sums<RB>(s_val, 1, r + (int64_t)blockIdx.x * kRunRegion);
     }
     grid_arrive(g, epoch);
@@ -1741,7 +1775,7 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     // ---- reorthogonalization of v_i and f against V_{<i} (classical Gram-Schmidt, `passes` times) ----
     double inv = 0.0, svf = 0.0;   // 1 / ||v_i|| and v_i^H f of the normalization
     for (int pass = 0;; ++pass) {
-      rows_times_h<RB>(sV, kcap, s_hl, b.V, ldv, row0, rows, k, H, s_sub, s_red, s_tail, s_he);
+      rows_times_h<RB>(sV, s_ve, kcap, s_hl, b.V, ldv, row0, rows, k, H, s_sub, s_red, s_tail, s_he);
       if (own) {
         const double sv = s_sub[0][threadIdx.x], sf = s_sub[1][threadIdx.x];
         v -= sv;
@@ -1754,7 +1788,7 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
       }
       if (passes > 1) {
         stage_y(v, f);
-        col_dots<RB>(sV, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
+        col_dots<RB>(sV, s_ve, kcap, b.V, ldv, row0, rows, k, s_y, s_yl, s_ye, hpart);
       } else {
         __syncthreads();
       }
@@ -1773,7 +1807,6 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     // and ||f||^2 from one sum (the readers of f subtract) ----
     v = inv * v;
     f = fma(-(svf * inv), v, f);
-    keep(k, v);
     if (own) {
       vi[e] = v;
       fn[e] = f;
@@ -1781,9 +1814,11 @@ __global__ void __launch_bounds__(RT) k_seed_run_csr_reorth(SeedBufs<double> b, 
     if ((int)threadIdx.x < RB) {
       s_val[0][threadIdx.x] = own ? f * f : 0.0;
       s_val[1][threadIdx.x] = own ? v * f : 0.0;
+      s_y[0][threadIdx.x] = own ? v : 0.0;
     }
     r = region();
     __syncthreads();
+    keep(k);
     row_sums<RB>(s_val, 2, r + (int64_t)blockIdx.x * kRunRegion);
     if (!grid_sync(g, epoch)) return;
     gather(nullptr, 0, nullptr, r, 2, s_sum);
@@ -2393,11 +2428,11 @@ static const void *reorth_run_kernel(int rb) {
 }
 // columns of V whose rows a block keeps in shared memory, and the bytes they take
 static int reorth_run_cols(int rb, int m) {
-  const int most = kRunSmem / ((rb + 1) * (int)sizeof(int2) + (int)sizeof(int4));
+  const int most = kRunSmem / ((rb + 1) * (int)sizeof(int2) + (int)sizeof(int4) + (int)sizeof(int));
   return m < most ? m : most;
 }
 static size_t reorth_run_smem(int rb, int kcap) {
-  return (size_t)kcap * ((rb + 1) * sizeof(int2) + sizeof(int4));
+  return (size_t)kcap * ((rb + 1) * sizeof(int2) + sizeof(int4) + sizeof(int));
 }
 
 int reorth_run_grid_cap(int sm_count, int rb) {
