@@ -633,7 +633,7 @@ int cg_csr_grid(const seed_ctx *ctx, int nc) {
 // The one-launch seed run and lockstep CG of small real CSR problems: rows per
 // block, the smallest of 16, 32, 64 whose grid has no more blocks than there are
 // SMs (a barrier of 256 blocks takes 4.2 us, of 128 blocks 3.1 us) or, failing that,
-// than can be resident; grid 0 when the problem does not qualify.
+// than can be resident (only on fewer than 152 SMs); grid 0 when the problem does not qualify.
 struct ReorthRun {
   int rb = 0, grid = 0;
 };
@@ -675,7 +675,8 @@ seed_status seed_reorth_run(seed_ctx *ctx, int nrhs, ReorthRun shape) {
   CU(cudaMemsetAsync(ctx->gsync, 0, sizeof(unsigned) * kGridSyncWords, ctx->cs));
   cudaError_t e = launch_seed_run_csr_reorth(b, ctx->csr, (double *)ctx->f2, g, ctx->partials, ctx->rhpart,
                                              reinterpret_cast<double *>(ctx->H), p.reorth_freq, p.reorth_passes,
-                                             p.m_max + 1, shape.rb, shape.grid, ctx->cs);
+                                             p.m_max + 1, shape.rb, shape.grid,
+                                             ctx->in_batch || shape.grid > ctx->sm_count, ctx->cs);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, SEED_ECUDA, std::string("persistent seed launch: ") + cudaGetErrorString(e));

@@ -1325,7 +1325,6 @@ __global__ void __launch_bounds__(CRT) k_seed_run_csr(SeedBufs<T> b, CsrOpT<T> o
 constexpr int kRunRegion = 32;                 // doubles per block in a scalar partial region
 constexpr int kRunMaxRhs = kReorthRunMaxRhs;   // alpha_i and g^2..g^16 in one region row
 constexpr int RT = 256;                        // threads per block
-constexpr int kRunSmem = 100 * 1024;           // shared memory of V's rows and H: two problems' blocks fit an SM
 // V's rows of a block by column, the block's v_i / u / f, H 2^(its column's exponent): |I| <= 2^kBits.
 // Bounds: |hi| <= 2^28, |lo| <= 2^27, so a sum of up to 64 products has |hi hi| parts below 2^62, cross
 // terms too; 50 or more columns per thread do not fit in shared memory.
@@ -1480,8 +1479,7 @@ SEED_DEV void col_dots(const int2 *sV, const int *ve, int kcap, const double *V,
 // as limbs with one exponent per v, into s_hl.
 template <int RB>
 SEED_DEV void rows_times_h(const int2 *sV, const int *ve, int kcap, int4 *s_hl, const double *V, int64_t ldv, int64_t row0, int rows,
-                           int k, const double *H, double (*sub)[RB], long long (*sred)[2 * RB], double (*stail)[2 * RB],
-                           int (*s_he)[2]) {
+                           int k, const double *H, double (*sub)[RB], long long (*sred)[2 * RB], int (*s_he)[2]) {
   constexpr int kGroups = RT / RB;
   const int kf = k < kcap ? k : kcap;   // columns in shared memory
   int e0 = -3000, e1 = -3000;   // below any sum of two exponents
@@ -1526,8 +1524,21 @@ SEED_DEV void rows_times_h(const int2 *sV, const int *ve, int kcap, int4 *s_hl, 
   }
   sred[grp][r] = limb_carry(a0, m0);
   sred[grp][RB + r] = limb_carry(a1, m1);
-  const bool tail = k > kf;
-  if (tail) {
+  __syncthreads();
+  const int q = threadIdx.x;   // < 2 RB: this thread's output
+  double d = 0.0;
+  if (q < 2 * RB) {
+    long long t = 0;   // the groups' sums in two parts: all of them could pass 63 bits
+    int lo = 0;
+#pragma unroll
+    for (int g2 = 0; g2 < kGroups; ++g2) {
+      t += sred[g2][q] >> 8;
+      lo += (int)(sred[g2][q] & 255);
+    }
+    d = scalbn(fma((double)t, 256.0, (double)lo), 56 - 2 * kBits + (q < RB ? e0 : e1));
+  }
+  if (k > kf) {   // the columns that are not in shared memory
+    double (*stail)[2 * RB] = reinterpret_cast<double (*)[2 * RB]>(sred);
     double pv = 0.0, pf = 0.0;
     if (r < rows) {
       const double *vr = V + row0 + r;
@@ -1537,24 +1548,14 @@ SEED_DEV void rows_times_h(const int2 *sV, const int *ve, int kcap, int4 *s_hl, 
         pf = fma(x, __ldcg(H + 2 * c + 1), pf);
       }
     }
+    __syncthreads();
     stail[grp][r] = pv;
     stail[grp][RB + r] = pf;
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < 2 * RB) {
-    const int q = threadIdx.x;
-    long long t = 0;   // the groups' sums in two parts: all of them could pass 63 bits
-    int lo = 0;
-#pragma unroll
-    for (int g2 = 0; g2 < kGroups; ++g2) {
-      t += sred[g2][q] >> 8;
-      lo += (int)(sred[g2][q] & 255);
-    }
-    double d = scalbn(fma((double)t, 256.0, (double)lo), 56 - 2 * kBits + (q < RB ? e0 : e1));
-    if (tail)
+    __syncthreads();
+    if (q < 2 * RB)
       for (int g2 = 0; g2 < kGroups; ++g2) d += stail[g2][q];
-    sub[q / RB][q % RB] = d;
   }
+  if (q < 2 * RB) sub[q / RB][q % RB] = d;
   __syncthreads();
 }
 
@@ -1563,7 +1564,10 @@ __global__ void __launch_bounds__(RT, 2) k_seed_run_csr_reorth(SeedBufs<double> 
                                                             double *bpart, double *hpart, double *H, int freq,
                                                             int passes, int i_stop, int kcap) {
   static_assert(2 * RB <= RT && RT % RB == 0, "rows per block");
-  __shared__ double s_val[kRunMaxRhs][RB];
+  // the values of row_sums and the group sums of rows_times_h, at different times
+  __shared__ double s_work[kRunMaxRhs * RB > 2 * RT ? kRunMaxRhs * RB : 2 * RT];
+  double (*const s_val)[RB] = reinterpret_cast<double (*)[RB]>(s_work);
+  long long (*const s_red)[2 * RB] = reinterpret_cast<long long (*)[2 * RB]>(s_work);
   __shared__ double s_sum[kRunRegion];
   __shared__ double2 s_g[kRunMaxRhs];
   __shared__ double2 s_eta[kRunMaxRhs];
@@ -1571,8 +1575,6 @@ __global__ void __launch_bounds__(RT, 2) k_seed_run_csr_reorth(SeedBufs<double> 
   __shared__ int4 s_yl[RB];
   __shared__ int s_ye[2], s_he[RT / 32][2];
   __shared__ double s_sub[2][RB];
-  __shared__ long long s_red[RT / RB][2 * RB];
-  __shared__ double s_tail[RT / RB][2 * RB];
   __shared__ LocalSeed L;
   extern __shared__ int4 s_run[];
   int4 *const s_hl = s_run;                                  // [kcap] limbs of H
@@ -1775,7 +1777,7 @@ __global__ void __launch_bounds__(RT, 2) k_seed_run_csr_reorth(SeedBufs<double> 
     // ---- reorthogonalization of v_i and f against V_{<i} (classical Gram-Schmidt, `passes` times) ----
     double inv = 0.0, svf = 0.0;   // 1 / ||v_i|| and v_i^H f of the normalization
     for (int pass = 0;; ++pass) {
-      rows_times_h<RB>(sV, s_ve, kcap, s_hl, b.V, ldv, row0, rows, k, H, s_sub, s_red, s_tail, s_he);
+      rows_times_h<RB>(sV, s_ve, kcap, s_hl, b.V, ldv, row0, rows, k, H, s_sub, s_red, s_he);
       if (own) {
         const double sv = s_sub[0][threadIdx.x], sf = s_sub[1][threadIdx.x];
         v -= sv;
@@ -2426,20 +2428,38 @@ static const void *reorth_run_kernel(int rb) {
   return rb == 16 ? (const void *)k_seed_run_csr_reorth<16> : rb == 32 ? (const void *)k_seed_run_csr_reorth<32>
                                                                        : (const void *)k_seed_run_csr_reorth<64>;
 }
-// columns of V whose rows a block keeps in shared memory, and the bytes they take
-static int reorth_run_cols(int rb, int m) {
-  const int most = kRunSmem / ((rb + 1) * (int)sizeof(int2) + (int)sizeof(int4) + (int)sizeof(int));
-  return m < most ? m : most;
+// Bytes of shared memory for a block's rows of V and for H, so that the blocks of two problems (a batch) fit
+// an SM together: half an SM's, without the kernel's own and the system's share (101 to 108 KB).  Two 64 x 64
+// Laplacians in a batch 14.7 -> 9.3 ms, two of 96 x 96 35.2 -> 22.5 (the 32 and 64 row forms did not fit twice).
+static int reorth_run_room_of(int rb) {
+  cudaFuncAttributes a;
+  int dev = 0, sm = 0, sys = 0;
+  if (cudaFuncGetAttributes(&a, reorth_run_kernel(rb)) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sys, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  const int room = sm / 2 - sys - (int)a.sharedSizeBytes;
+  return room > 0 ? room / 128 * 128 : 0;
 }
-static size_t reorth_run_smem(int rb, int kcap) {
-  return (size_t)kcap * ((rb + 1) * sizeof(int2) + sizeof(int4) + sizeof(int));
+static int reorth_run_room(int rb) {
+  static const int room[3] = {reorth_run_room_of(16), reorth_run_room_of(32), reorth_run_room_of(64)};
+  return room[rb >> 5];
 }
+// What a block that has its SM to itself asks for: more than half an SM's, so that a kernel alone on the GPU keeps
+// more L1 (64 x 64 Laplacian 8.27 ms instead of 8.37; with the same columns either way).
+static int reorth_run_most(int rb) { return reorth_run_room(rb) + 4096; }
+static size_t reorth_run_column(int rb) { return (rb + 1) * sizeof(int2) + sizeof(int4) + sizeof(int); }
+// columns of V whose rows a block keeps there
+static int reorth_run_cols(int rb, int m) { return std::min(m, reorth_run_room(rb) / (int)reorth_run_column(rb)); }
 
 int reorth_run_grid_cap(int sm_count, int rb) {
   int per_sm = 0;
   const void *k = reorth_run_kernel(rb);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunSmem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, RT, kRunSmem) != cudaSuccess) {
+  const int room = reorth_run_room(rb);
+  if (room == 0 || cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, reorth_run_most(rb)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, RT, room) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -2449,12 +2469,13 @@ int reorth_run_grid_cap(int sm_count, int rb) {
 
 cudaError_t launch_seed_run_csr_reorth(const SeedBufs<double> &b, const CsrOp &op, double *f2, GridSync g,
                                        double *bpart, double *hpart, double *H, int freq, int passes, int i_stop,
-                                       int rb, int grid, cudaStream_t s) {
+                                       int rb, int grid, bool share, cudaStream_t s) {
   SeedBufs<double> bb = b;
   CsrOp o = op;
   int kcap = reorth_run_cols(rb, i_stop);
+  const size_t most = reorth_run_most(rb);
   void *args[] = {&bb, &o, &f2, &g, &bpart, &hpart, &H, &freq, &passes, &i_stop, &kcap};
-  return cudaLaunchCooperativeKernel(reorth_run_kernel(rb), dim3(grid), dim3(RT), args, reorth_run_smem(rb, kcap), s);
+  return cudaLaunchCooperativeKernel(reorth_run_kernel(rb), dim3(grid), dim3(RT), args, share ? kcap * reorth_run_column(rb) : most, s);
 }
 
 cudaError_t launch_cg_run_csr(const CsrOp &op, const CallArgs *call, double *R, double *P, double *Q, int64_t ld,
