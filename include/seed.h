@@ -312,7 +312,9 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
  * cudaMalloc had run out of memory, without calling it; the call that needed
  * it returns SEED_ENOMEM.  A failed seed_create_* frees what it had
  * allocated; a failed call on a context leaves the context valid, and a later
- * call allocates what is still missing.  k <= 0 disarms.  Process-wide (all
+ * call allocates what is still missing.  Work space that a call can do without (the
+ * fixed-point Wilson operator's) is not counted: where cudaMalloc has no room for it, the
+ * call runs in FP64 arithmetic.  k <= 0 disarms.  Process-wide (all
  * threads and contexts).  Returns the previous countdown.
  *
  * seed_check_barrier_timeout: self-test of the bounded wait of the persistent

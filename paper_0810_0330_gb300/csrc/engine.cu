@@ -68,12 +68,14 @@ struct seed_ctx {
   CsrOp csr{};
   WilsonOp wil{};
   int32_t *nbr = nullptr;
-  // Wilson: the FP64 operator in fixed-point arithmetic (wilson_fixed.cuh).  flinks / fexp are
-  // filled from the caller's links by every call that applies the operator; F and T hold the
-  // blocks of A's input and of D's output, Fe their exponents (F's columns, then T's).
+  // Wilson: the FP64 operator in fixed-point arithmetic (wilson_fixed.cuh).  flinks / fexp (one
+  // allocation) are filled from the caller's links by every call that uses this form; F and T hold
+  // the blocks of A's input and of D's output, Fe (behind F) their exponents (F's columns, then T's).
+  // All of it, and dotpart, is allocated by the first call that uses it, and a call that gets no
+  // memory for it runs in FP64 arithmetic (ensure_fixed).
   WilsonFix wfix{};
   int4 *flinks = nullptr, *F = nullptr;
-  int32_t *fexp = nullptr, *Fe = nullptr;
+  int32_t *Fe = nullptr;
   bool links_ready = false;            // flinks hold the links of the current call
   double *dotpart = nullptr;           // partial sums of p^H q by 16 sites (wilson_fixed.cu)
 
@@ -227,6 +229,25 @@ seed_status dalloc(seed_ctx *ctx, Tp **p, size_t bytes) {
   return SEED_OK;
 }
 
+// Work space that a call can do without: false where there is no memory (no failure of the call,
+// and not counted by seed_inject_alloc_failure).  Also inside a capture on the caller's stream,
+// where an allocation is allowed in the relaxed mode only.
+template <class Tp>
+bool dalloc_spare(Tp **p, size_t bytes) {
+  if (*p) return true;
+  void *q = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaMalloc(&q, bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  *p = reinterpret_cast<Tp *>(q);
+  return true;
+}
+
 #define TRY(x)                        \
   do {                                \
     seed_status s_ = (x);             \
@@ -308,7 +329,7 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
   if (cols <= ctx->cap_cols) return SEED_OK;
   cudaStreamSynchronize(ctx->cs);
   cudaEventSynchronize(ctx->ev_apply);
-  for (void *q : {ctx->T, (void *)ctx->F, (void *)ctx->Fe, ctx->P32, ctx->T32}) {
+  for (void *q : {ctx->T, (void *)ctx->F, ctx->P32, ctx->T32}) {
     if (ctx->captured && q) ctx->kept.push_back(q);   // a replay may still come
     else cudaFree(q);
   }
@@ -318,6 +339,7 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
   ctx->F = nullptr;
   ctx->Fe = nullptr;
   ctx->dotpart = nullptr;
+  ctx->links_ready = false;
   cudaFree(ctx->R32); cudaFree(ctx->Q32); cudaFree(ctx->E32);
   ctx->R32 = ctx->P32 = ctx->Q32 = ctx->T32 = ctx->E32 = nullptr;
   ctx->cap_cols = 0;
@@ -341,29 +363,29 @@ seed_status ensure_cols(seed_ctx *ctx, int cols) {
   return SEED_OK;
 }
 
-// What the fixed-point operator needs, for a call that uses it (never inside a graph capture): its
-// work space for the context's columns, and the copy of the caller's links, once per call (the
-// caller may have changed them since the last one).
-seed_status ensure_fixed(seed_ctx *ctx, bool links = true) {
-  if (ctx->kind != 1 || ctx->links_ready) return SEED_OK;
-  const size_t cols = ctx->cap_cols;
-  if (!ctx->F) TRY(dalloc(ctx, &ctx->F, (size_t)ctx->ldv * cols * sizeof(int4)));
-  if (!ctx->Fe) TRY(dalloc(ctx, &ctx->Fe, sizeof(int32_t) * 2 * (size_t)(ctx->ldv / 12) * cols));
-  if (!ctx->dotpart) TRY(dalloc(ctx, &ctx->dotpart, sizeof(double) * (size_t)(ctx->ldv / 192) * cols));
-  if (!links) return SEED_OK;
+// What the fixed-point operator needs: work space for the context's columns (false: no memory) ...
+bool fix_space(seed_ctx *ctx) {
+  const int64_t tiles = (ctx->wfix.sites + 31) / 32;
+  const size_t cols = ctx->cap_cols, f = (size_t)ctx->ldv * cols * sizeof(int4);
+  if (!dalloc_spare(&ctx->flinks, sizeof(int4) * 4 * 288 * (size_t)tiles + sizeof(int32_t) * 4 * (size_t)ctx->wfix.sites))
+    return false;
+  ctx->wfix.flinks = ctx->flinks;
+  ctx->wfix.fexp = reinterpret_cast<int32_t *>(ctx->flinks + 4 * 288 * tiles);
+  if (!dalloc_spare(&ctx->F, f + sizeof(int32_t) * 2 * (size_t)(ctx->ldv / 12) * cols)) return false;
+  ctx->Fe = reinterpret_cast<int32_t *>(ctx->F + (size_t)ctx->ldv * cols);
+  return true;
+}
+// ... and the copy of the caller's links, once per call (the caller may have changed them since the last
+// one).  A call whose ensure_fixed got no memory finds links_ready false and applies the FP64 kernels.
+void ensure_fixed(seed_ctx *ctx) {
+  if (ctx->kind != 1 || ctx->links_ready || !fix_space(ctx)) return;
   launch_fix_links(ctx->wfix, ctx->cs);
   ctx->links_ready = true;
   ctx->stats.kernel_launches += 1;
-  return SEED_OK;
 }
-
-// The same for the operator by itself: false (the caller takes the FP64 kernel, which needs no work
-// space) where an allocation fails or a capture of the caller's stream forbids it.
-bool try_fixed(seed_ctx *ctx, bool links) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (!ctx->F || !ctx->Fe || !ctx->dotpart)
-    if (cudaStreamIsCapturing(ctx->cs, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
-  return ensure_fixed(ctx, links) == SEED_OK;
+// Partial sums of p^H q for the operators that form alpha (false: no memory).
+bool dot_space(seed_ctx *ctx) {
+  return dalloc_spare(&ctx->dotpart, sizeof(double) * (size_t)(ctx->ldv / 192) * ctx->cap_cols);
 }
 
 // T's columns hold blocks (16 bytes per component, like its doubles); Te: their exponents
@@ -378,6 +400,7 @@ int32_t *fix_Te(seed_ctx *ctx) { return ctx->Fe + ctx->ldv / 12 * ctx->cap_cols;
 // x 16, 5e-14 on 12^4 and below 1e-13 on 16^4; so from kFixSeedSites on they take the
 // fixed-point operator (apply_seed).
 constexpr int64_t kFixSeedSites = 16384;
+bool fix_seed(const seed_ctx *ctx) { return ctx->kind == 1 && ctx->wfix.sites >= kFixSeedSites; }
 int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols) {
   if (ctx->kind == 0) {
     launch_csr_spmv(ctx->csr, (const double *)X, ldx, (double *)Y, ldy, ncols, nullptr, ctx->cs);
@@ -392,7 +415,6 @@ int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, i
 // Wilson: in fixed-point arithmetic from one tile per SM on; below that the FP64 kernel's two
 // launches (one tile's FP64 instructions on its SM) are the shorter chain than four, and
 // seed_apply converts links and spinors in one.
-bool fix_seed(const seed_ctx *ctx) { return ctx->kind == 1 && ctx->wfix.sites >= kFixSeedSites; }
 bool fix_pays(const seed_ctx *ctx, int ncols) { return ctx->kind == 1 && ctx->ldv / 384 * ncols > ctx->sm_count; }
 int apply_A(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols, const int32_t *mask) {
   if (ctx->kind == 0) {
@@ -571,7 +593,8 @@ int issue_seed_step(seed_ctx *ctx, int nrhs, bool reorth) {
 // Capture (once) and launch a graph for the given pattern of steps.
 template <class T>
 seed_status launch_seed_run(seed_ctx *ctx, int nrhs, const std::vector<char> &pattern) {
-  std::string key = (kLow<T> ? "s" : "S") + std::to_string(nrhs) + ":" + std::string(pattern.begin(), pattern.end());
+  std::string key = (kLow<T> ? "s" : ctx->links_ready ? "Sf" : "S") + std::to_string(nrhs) + ":" +
+                    std::string(pattern.begin(), pattern.end());
   auto it = ctx->graphs.find(key);
   if (it == ctx->graphs.end()) {
     GraphEntry g;
@@ -616,10 +639,11 @@ int csr_seed_grid(const seed_ctx *ctx) {
 // thread per site; 16^3 x 32 mixed seed phase 40.1 ms from graphs of step
 // kernels, 37.1 ms in the site form).  Not in FP64 from kFixSeedSites on: there
 // step kernels with the fixed-point operator beat the run's FP64 tiles (16^4, 303
-// steps: 176 -> 95 ms).
+// steps: 176 -> 95 ms), unless its work space could not be had.
 bool use_persistent_seed(seed_ctx *ctx) {
   const int f = ctx->prm.reorth_freq;
-  return ctx->allow_persistent && ctx->pgrid > 0 && (f == 0 || f >= 8) && !(ctx->precision == 0 && fix_seed(ctx));
+  return ctx->allow_persistent && ctx->pgrid > 0 && (f == 0 || f >= 8) &&
+         !(ctx->precision == 0 && fix_seed(ctx) && ctx->links_ready);
 }
 
 // Blocks of the persistent CSR CG: one per work item (1024 rows of one column)
@@ -774,7 +798,7 @@ seed_status solve_first_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
   const int64_t n = ctx->n;
   const seed_params &p = ctx->prm;
   TRY(ensure_cols(ctx, std::max(nrhs, 1)));
-  TRY(ensure_fixed(ctx));
+  if (fix_seed(ctx)) ensure_fixed(ctx);
   if (blocked_seeding(ctx, nrhs)) TRY(ensure_block(ctx));
   ctx->basis_valid = false;
   ctx->seeded = false;
@@ -869,12 +893,30 @@ seed_status solve_first_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
 
 // One lockstep CG iteration on the CG columns c0 .. c0 + c.nc - 1 (c: the view
 // of those columns), on stream s, with its own CallArgs slot, partials and
-// tickets (two branches of a graph run at the same time on disjoint columns).
+// tickets (two branches of a graph run at the same time on disjoint columns).  fixed: the
+// Wilson operator in fixed-point arithmetic.
 template <class T>
 int issue_cg_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, const CallArgs *call, double *partials,
-                  unsigned *tickets) {
+                  unsigned *tickets, bool fixed) {
   const int64_t n = ctx->n, ld = ctx->ldv;
   T *P = (T *)ctx->P + (int64_t)c0 * ld, *Q = (T *)ctx->Q + (int64_t)c0 * ld, *R = (T *)ctx->R + (int64_t)c0 * ld;
+  int k = 1;
+  if constexpr (std::is_same_v<T, double2>) {
+    if (!fixed) {   // no memory for the blocks
+      double2 *Tb = (double2 *)ctx->T + (int64_t)c0 * ld;
+      launch_wilson_dslash(ctx->wil, +1, P, ld, Tb, ld, c.nc, c.active, s);
+      launch_wilson_dslash(ctx->wil, -1, Tb, ld, Q, ld, c.nc, c.active, s);
+      k = 2;
+    }
+  } else {
+    launch_csr_spmv(ctx->csr, P, ld, Q, ld, c.nc, c.active, s);
+  }
+  if (!fixed) {
+    launch_cg_alpha<T>(n, P, Q, ld, c, partials, tickets, s);
+    launch_cg_residual<T>(n, R, Q, ld, c, partials, tickets, s);
+    launch_cg_xp<T>(n, call, R, P, ld, c, s);
+    return k + 3;
+  }
   if constexpr (std::is_same_v<T, double2>) {
     // p's blocks are in F: t = D p, q = D^H t with alpha, the residual, then x and p (with its blocks)
     int4 *Fb = ctx->F + (int64_t)c0 * ld, *Tb = fix_T(ctx) + (int64_t)c0 * ld;
@@ -884,14 +926,8 @@ int issue_cg_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, const 
     launch_dslash_fix(ctx->wfix, -1, Tb, Te, ld, nullptr, nullptr, Q, ld, c.nc, c.active, s, &dot);
     launch_cg_residual<T>(n, R, Q, ld, c, partials, tickets, s);
     launch_cg_xp_fix(ctx->wfix, call, R, P, ld, Fb, Fe, c, s);
-    return 4;
-  } else {
-    launch_csr_spmv(ctx->csr, P, ld, Q, ld, c.nc, c.active, s);
-    launch_cg_alpha<T>(n, P, Q, ld, c, partials, tickets, s);
-    launch_cg_residual<T>(n, R, Q, ld, c, partials, tickets, s);
-    launch_cg_xp<T>(n, call, R, P, ld, c, s);
-    return 4;
   }
+  return 4;
 }
 
 // The columns c0 .. c0 + nc - 1 of the per-column CG state.
@@ -1000,15 +1036,15 @@ seed_status read_cg(seed_ctx *ctx, CgHost *h) {
 }
 
 template <class T>
-seed_status launch_cg_run(seed_ctx *ctx, const CgCols &c, int len) {
-  std::string key = "C" + std::to_string(c.nc) + ":" + std::to_string(len);
+seed_status launch_cg_run(seed_ctx *ctx, const CgCols &c, int len, bool fixed) {
+  std::string key = (fixed ? "Cf" : "C") + std::to_string(c.nc) + ":" + std::to_string(len);
   auto it = ctx->graphs.find(key);
   if (it == ctx->graphs.end()) {
     GraphEntry g;
     cudaGraph_t graph;
     CU(cudaStreamBeginCapture(ctx->cs, cudaStreamCaptureModeThreadLocal));
     g.kernels += issue_cg_branches(ctx, c, len, cg_most(ctx, c.nc), [&](const CgCols &v, int c0, cudaStream_t s, int b) {
-      return issue_cg_iter<T>(ctx, v, c0, s, ctx->call + b, branch_partials(ctx, b), ctx->tickets + c0);
+      return issue_cg_iter<T>(ctx, v, c0, s, ctx->call + b, branch_partials(ctx, b), ctx->tickets + c0, fixed);
     });
     CU(cudaStreamEndCapture(ctx->cs, &graph));
     cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
@@ -1038,18 +1074,19 @@ seed_status cg_impl(seed_ctx *ctx, const T *Bc, int64_t ldb, T *Xc, int64_t ldx,
   for (int b = 0; b < nb; ++b) ca[b] = CallArgs{Xc, ldx, start[b]};
   CU(cudaMemcpyAsync(ctx->call, ca, sizeof(CallArgs) * nb, cudaMemcpyHostToDevice, ctx->cs));
   const CgCols c = cg_cols(ctx, nc);
-  TRY(ensure_fixed(ctx));
+  ReorthRun scg;   // small real CSR problems: the one-launch CG with two barriers per iteration
+  if constexpr (std::is_same_v<T, double>) scg = small_cg_shape(ctx, nc);
+  const bool persist = scg.grid > 0 || (ctx->allow_persistent_cg && ctx->pgrid_cg > 0 && nc <= kPersistMaxCols);
+  if (!persist || fix_pays(ctx, nc)) ensure_fixed(ctx);
+  const bool fixed = !persist && ctx->links_ready && dot_space(ctx);
   // K7: true residual of the seeded systems, then p = r
   int kern = apply_A(ctx, Xc, ldx, ctx->Q, ld, nc, nullptr);
   launch_cg_init<T>(n, Bc, ldb, (const T *)ctx->Q, ld, (T *)ctx->R, (T *)ctx->P, ld, c, ctx->partials, ctx->tickets,
                     false, ctx->cs);
   ctx->stats.kernel_launches += kern + 1;
   ctx->stats.mvps += nc;
-  ReorthRun scg;   // small real CSR problems: the one-launch CG with two barriers per iteration
-  if constexpr (std::is_same_v<T, double>) scg = small_cg_shape(ctx, nc);
-  const bool persist = scg.grid > 0 || (ctx->allow_persistent_cg && ctx->pgrid_cg > 0 && nc <= kPersistMaxCols);
-  auto blocks_of_p = [&]() {   // Wilson: p's fixed-point blocks, kept up by the iterations from here on
-    if (ctx->kind != 1 || persist) return;
+  auto blocks_of_p = [&]() {   // p's fixed-point blocks, kept up by the iterations from here on
+    if (!fixed) return;
     launch_fix_spinors(ctx->wfix, (const double2 *)ctx->P, ld, ctx->F, ld, ctx->Fe, nc, c.active, ctx->cs);
     ctx->stats.kernel_launches += 1;
   };
@@ -1084,7 +1121,7 @@ seed_status cg_impl(seed_ctx *ctx, const T *Bc, int64_t ldb, T *Xc, int64_t ldx,
       int slot = 0, pending = -1;
       cudaEvent_t evs[2] = {nullptr, nullptr};
       for (;;) {
-        TRY(launch_cg_run<T>(ctx, c, L));
+        TRY(launch_cg_run<T>(ctx, c, L, fixed));
         CU(cudaMemcpyAsync(ctx->h_flags + slot * kMaxRhs, c.active, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost,
                            ctx->cs));
         if (!evs[slot]) CU(cudaEventCreateWithFlags(&evs[slot], cudaEventDisableTiming));
@@ -1249,8 +1286,8 @@ seed_status solve_related_impl(seed_ctx *ctx, const void *B, int64_t ldb, void *
   if (info && nc > 0) std::memset(info + 1, 0, sizeof(seed_info) * nc);
   if (nc <= 0) return SEED_OK;
   TRY(ensure_cols(ctx, nrhs));
-  TRY(ensure_fixed(ctx));
   TRY(ensure_related(ctx, nc));
+  if (fix_pays(ctx, nc)) ensure_fixed(ctx);
   const T *Bt = (const T *)B;
   T *Xt = (T *)X;
   T *R = (T *)ctx->Rrel, *xb = (T *)ctx->xrel, *rb = (T *)ctx->rrel;
@@ -1326,7 +1363,7 @@ seed_status solve_multiple_impl(seed_ctx *ctx, const void *B, int64_t ldb, void 
   c.max_restarts = 0;
   c.tol_check = 1.5 * c.tol;
   const int L = 16;
-  TRY(ensure_fixed(ctx));
+  if (fix_pays(ctx, 1)) ensure_fixed(ctx);
   for (int j = 0; j < nrhs; ++j) {
     const CallArgs ca{Xw, ld, j};
     CU(cudaMemcpyAsync(ctx->call, &ca, sizeof(ca), cudaMemcpyHostToDevice, ctx->cs));
@@ -1335,7 +1372,7 @@ seed_status solve_multiple_impl(seed_ctx *ctx, const void *B, int64_t ldb, void 
                       ctx->partials, ctx->tickets, false, ctx->cs);
     ctx->stats.kernel_launches += kern + 1;
     const int nrem = nrhs - j - 1;
-    const std::string key = "MS" + std::to_string(nrhs) + ":" + std::to_string(j) + ":" + std::to_string(L);
+    const std::string key = (ctx->links_ready ? "MSf" : "MS") + std::to_string(nrhs) + ":" + std::to_string(j) + ":" + std::to_string(L);
     int slot = 0, pending = -1;
     cudaEvent_t evs[2] = {nullptr, nullptr};
     for (;;) {
@@ -1433,18 +1470,20 @@ int issue_mixed_iter(seed_ctx *ctx, const CgCols &c, int c0, cudaStream_t s, con
   const int64_t n = ctx->nv, ld = ctx->ldv;
   T32 *P = (T32 *)ctx->P32 + (int64_t)c0 * ld, *Q = (T32 *)ctx->Q32 + (int64_t)c0 * ld;
   T32 *R = (T32 *)ctx->R32 + (int64_t)c0 * ld;
+  bool alpha = false;   // formed by D^H
   if constexpr (std::is_same_v<T32, float>) {
     launch_csr_spmv32(ctx->csr32, P, ld, Q, ld, c.nc, c.active, s);
-    launch_cg_alpha<T32>(n, P, Q, ld, c, partials, tickets, s);
   } else {
     float2 *Tb = (float2 *)ctx->T32 + (int64_t)c0 * ld;
-    const CgDot<float2> dot{P, ctx->dotpart + (int64_t)c0 * (ld / 192), tickets, c.rho, c.alpha};
+    alpha = ctx->dotpart != nullptr;
+    const CgDot<float2> dot{P, alpha ? ctx->dotpart + (int64_t)c0 * (ld / 192) : nullptr, tickets, c.rho, c.alpha};
     launch_wilson_dslash32(ctx->wil32, +1, P, ld, Tb, ld, c.nc, c.active, true, s);
-    launch_wilson_dslash32(ctx->wil32, -1, Tb, ld, Q, ld, c.nc, c.active, true, s, &dot);
+    launch_wilson_dslash32(ctx->wil32, -1, Tb, ld, Q, ld, c.nc, c.active, true, s, alpha ? &dot : nullptr);
   }
+  if (!alpha) launch_cg_alpha<T32>(n, P, Q, ld, c, partials, tickets, s);
   launch_cg_residual<T32>(n, R, Q, ld, c, partials, tickets, s);
   launch_cg_xp<T32>(n, call, R, P, ld, c, s);
-  return 4;
+  return (ctx->kind == 1 ? 4 : 3) + !alpha;
 }
 
 // CG on columns c0..c0+nc-1 of B and X (FP64) to ||b - A x|| <= tol ||b||
@@ -1472,7 +1511,8 @@ seed_status mixed_cg(seed_ctx *ctx, const T64 *Bc, int64_t ldb, T64 *Xc, int64_t
   ctx->stats.mvps += nc;
   const int L = 16;
   // the graph bakes in CgCols (tolerance included): system 1 (c0 = 0) and the others have their own
-  const std::string key = "M" + std::to_string(nc) + ":" + std::to_string(L) + ":" + std::to_string(c0);
+  const bool dots = ctx->kind == 1 && dot_space(ctx);
+  const std::string key = (dots ? "Md" : "M") + std::to_string(nc) + ":" + std::to_string(L) + ":" + std::to_string(c0);
   int slot = 0, pending = -1;
   cudaEvent_t evs[2] = {nullptr, nullptr};
   for (;;) {
@@ -1518,7 +1558,7 @@ seed_status solve_first_mixed(seed_ctx *ctx, const void *B, int64_t ldb, void *X
   const int64_t n = ctx->n, ld = ctx->ldv;
   const seed_params &p = ctx->prm;
   TRY(ensure_cols(ctx, std::max(nrhs, 1)));
-  TRY(ensure_fixed(ctx));
+  if (fix_pays(ctx, nrhs)) ensure_fixed(ctx);
   if (blocked_seeding(ctx, nrhs)) TRY(ensure_block(ctx));
   ctx->basis_valid = false;
   ctx->seeded = false;
@@ -1631,7 +1671,7 @@ seed_status solve_rest_mixed(seed_ctx *ctx, const void *B, int64_t ldb, void *X,
   if (info) std::memset(info + 1, 0, sizeof(seed_info) * (nc > 0 ? nc : 0));
   if (nc <= 0) return SEED_OK;
   TRY(ensure_cols(ctx, nrhs));
-  TRY(ensure_fixed(ctx));
+  if (fix_pays(ctx, nc)) ensure_fixed(ctx);
   CU(cudaEventRecord(ctx->t2, ctx->cs));
   TRY((mixed_cg<T64, T32>(ctx, (const T64 *)B + ldb, ldb, (T64 *)X + ldx, ldx, 1, nc, ctx->prm.tol_rest, nullptr)));
   CU(cudaEventRecord(ctx->t3, ctx->cs));
@@ -1744,7 +1784,7 @@ void destroy(seed_ctx *ctx) {
   if (!ctx) return;
   if (ctx->cs) cudaStreamSynchronize(ctx->cs);
   if (ctx->ev_apply) cudaEventSynchronize(ctx->ev_apply);
-  cudaFree(ctx->flinks); cudaFree(ctx->fexp); cudaFree(ctx->F); cudaFree(ctx->Fe); cudaFree(ctx->dotpart);
+  cudaFree(ctx->flinks); cudaFree(ctx->F); cudaFree(ctx->dotpart);
   for (auto &kv : ctx->graphs) cudaGraphExecDestroy(kv.second.exec);
   void *ptrs[] = {ctx->V, ctx->u, ctx->f, ctx->w, ctx->st, ctx->alpha_hist, ctx->beta_hist,
                   ctx->delta_hist, ctx->eta, ctx->partials, ctx->tickets, ctx->Hpart, ctx->H, ctx->call,
@@ -1884,8 +1924,6 @@ seed_status seed_create_wilson(seed_ctx **out, const seed_wilson *A, const seed_
   ctx->nv = ctx->lay.length(ctx->n);
   s = alloc_common(ctx);
   if (s == SEED_OK) s = dalloc(ctx, &ctx->nbr, sizeof(int32_t) * 8 * vol);
-  if (s == SEED_OK) s = dalloc(ctx, &ctx->flinks, sizeof(int4) * 4 * 288 * (size_t)((vol + 31) / 32));
-  if (s == SEED_OK) s = dalloc(ctx, &ctx->fexp, sizeof(int32_t) * 4 * vol);
   if (s == SEED_OK && ctx->precision == 1) {
     const int64_t nl = 4 * vol * 9;
     s = dalloc(ctx, &ctx->op32, sizeof(float2) * (size_t)nl);
@@ -1909,8 +1947,6 @@ seed_status seed_create_wilson(seed_ctx **out, const seed_wilson *A, const seed_
     ctx->wfix.bc_t = A->bc_t;
     ctx->wfix.links = (const double2 *)A->links;
     ctx->wfix.nbr = ctx->nbr;
-    ctx->wfix.flinks = ctx->flinks;
-    ctx->wfix.fexp = ctx->fexp;
     for (int k = 0; k < 4; ++k) ctx->wil32.dims[k] = A->dims[k];
     ctx->wil32.sites = vol;
     ctx->wil32.kappa = A->kappa;
@@ -1963,8 +1999,8 @@ seed_status seed_solve_cg(seed_ctx *ctx, const void *B, int64_t ldb, void *X, in
   if (overlap(B, ldb, X, ldx, ncols, ctx->n, ctx->esz)) return fail(ctx, SEED_EINVAL, "B and X overlap");
   StreamScope scope(ctx);
   TRY(ensure_cols(ctx, ncols));
-  TRY(ensure_fixed(ctx));
   if (ctx->precision == 1) {
+    if (fix_pays(ctx, ncols)) ensure_fixed(ctx);
     if (info) std::memset(info, 0, sizeof(seed_info) * ncols);
     CU(cudaEventRecord(ctx->t2, ctx->cs));
     seed_status st;
@@ -2054,7 +2090,7 @@ seed_status seed_project(seed_ctx *ctx, const void *B, int64_t ldb, void *X, int
   if (overlap(B, ldb, X, ldx, ncols, ctx->n, ctx->esz)) return fail(ctx, SEED_EINVAL, "B and X overlap");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
-  if (!ctx->prm.x0_zero) TRY(ensure_fixed(ctx));
+  if (!ctx->prm.x0_zero && fix_pays(ctx, ncols)) ensure_fixed(ctx);
   const int64_t n = ctx->n, ld = ctx->ldv;
   int kern = 0;
   if (ctx->kind == 0) {
@@ -2109,7 +2145,8 @@ seed_status seed_apply(seed_ctx *ctx, int32_t op, const void *X, int64_t ldx, vo
   ApplyScope scope(ctx);
   const bool few = op == 0 && ctx->kind == 1 && !fix_pays(ctx, ncols);   // links and spinors converted in one launch
   // D and D^H in a capture take no work space: their graphs depend on the operator, X and Y alone
-  const bool fixed = ctx->kind == 1 && (op == 0 || (op < 3 && fix_seed(ctx) && !scope.capturing)) && try_fixed(ctx, !few);
+  const bool fixed = ctx->kind == 1 && (op == 0 || (op < 3 && fix_seed(ctx) && !scope.capturing)) && fix_space(ctx);
+  if (fixed && !few) ensure_fixed(ctx);
   if (scope.capturing && ctx->kind == 1 && (op == 0 || op == 3)) ctx->captured = true;
   if (op == 3) {
     ctx->stats.kernel_launches += apply_32(ctx, 0, X, ldx, Y, ldy, ncols, false);
@@ -2235,7 +2272,7 @@ seed_status seed_time_operator(seed_ctx *ctx, int32_t op, int32_t ncols, int32_t
   if (ncols < 1 || ncols > kMaxRhs || reps < 1 || reps > 100000) return fail(ctx, SEED_EINVAL, "bad ncols / reps");
   TRY(ensure_cols(ctx, ncols));
   StreamScope scope(ctx);
-  if (op == 0 && fix_pays(ctx, ncols)) TRY(ensure_fixed(ctx));
+  if (op == 0 && fix_pays(ctx, ncols)) ensure_fixed(ctx);
   CU(cudaMemsetAsync(ctx->P, 0x3F, (size_t)ctx->ldv * ncols * ctx->esz, ctx->cs));   // normal doubles ~4.8e-4
   if (op >= 3) CU(cudaMemsetAsync(ctx->P32, 0x3F, (size_t)ctx->ldv * ncols * ctx->vsz, ctx->cs));   // floats ~0.75
   // one untimed launch, then the timed ones
