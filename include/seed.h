@@ -297,6 +297,17 @@ seed_status seed_grad_kappa(seed_ctx *ctx, const void *Lambda, int64_t ldl, cons
  * 384 * ceil(sites / 32) (ldx, ldy >= that length); the padding sites of the
  * last tile are written as zeros.  X and Y must not overlap.  Runs on the
  * context's stream; not synchronising.
+ *   Accuracy of ops 0..2 on Wilson contexts.  Op 0, and ops 1 and 2 from 16384 sites on, run in
+ * fixed-point arithmetic on blocks of a site's 24 reals.  A result of D (D^H) has an error below
+ * 2^-46 of the largest term of its site: the largest real of x there, or |kappa| times a link's largest row
+ * or column sum of |Re| + |Im| times the largest real of x at that neighbour; on
+ * spinors whose components have similar sizes the error in the 2-norm is no larger than FP64
+ * arithmetic's (1.3e-16 of D^H D x).  That bound is by site, not by component: components much smaller than
+ * others at their site or its neighbours (decoupled colours or spins, e.g. in a free field)
+ * keep less relative accuracy than in FP64 arithmetic, or none below 2^-57 of the largest.
+ * Ops 1 and 2 in a stream capture, or below 16384 sites, and seed_wilson_apply_noalloc
+ * are in FP64 arithmetic (relative to the component's own terms), as is any op of these where
+ * there is no memory for the fixed-point form's work space.
  *   In a stream capture: the call needs room for ncols columns from an earlier
  * call; the graph is valid until seed_destroy.  Graphs of ops 1, 2, 4, 5, 6 and 7 (and of
  * ops 0 and 3 on a CSR context) use nothing but the operator, X and Y.  Graphs of ops 0 and 3 on a

@@ -20,10 +20,13 @@
 // 2^59 in units of 2^-58 2^(e+g), and eight hops plus the site's own term are
 // below 2^62.1: nothing can overflow 64 bits.  Each hop is shifted to the largest
 // exponent of the nine terms, E, before it is added, so the sum has an absolute
-// error of a few 2^-58 2^E, where FP64 arithmetic has rounding errors of 2^-54
-// of every partial sum.  Measured against 64-bit exact results, the relative
-// error of D^H D on random spinors is no larger than the FP64 kernel's (1.6e-16
-// before); tests/test_gpu_fixed.py holds it to that.
+// error of at most 269 units of 2^-58 2^E (per hop 12 for the dropped low products, 16 for
+// the link's rounding, 4 for the spinor's cut-off, 1.5 for the shifts), a few in practice, where FP64
+// arithmetic has rounding errors of 2^-54 of every partial sum.  In the 2-norm the error of D^H D on
+// random spinors is no larger than the FP64 kernel's (1.3e-16 against 1.6e-16;
+// tests/test_gpu_fixed.py holds it to that).  The bound is by site: a component far below its
+// site's largest term has less relative accuracy than in FP64 arithmetic, and none below 2^-57
+// of it (seed.h says so to the caller of seed_apply; tests/test_gpu_fixed_bound.py).
 //
 // Sites whose components are not finite, or whose largest one lies outside
 // 2^-700 .. 2^700, keep their doubles (exponent code kExpRaw), and a site with
