@@ -46,6 +46,11 @@ FP64_INSTR_PER_SITE_D = 816
 # FP64 peak from unit counts: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (the library's FMA-chain
 # probe, seed_time_fma, measures it live next to the roofline)
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07
+# The fixed-point operator of the FP64 CG: 32 x 32 -> 64 bit multiply-adds per site and column of D, 8 hops x
+# 2 half-spinor components x 9 complex products x 4 real products x 3 limb products
+INT_MADS_PER_SITE_D = 8 * 2 * 9 * 4 * 3
+# their rate, measured on this part: 61 per clock and SM (GMAD/s at 152 SMs and 2.07 GHz)
+INT_MAD_PEAK_G = 152 * 61 * 2.07
 try:
     with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as _fh:
         MEASURED_PEAKS = json.load(_fh)
@@ -480,42 +485,51 @@ def time_steps(S, torch, p, flush, steps, warmup, clk=None):
     return [a.elapsed_time(b) for a, b in ev], infos
 
 
-def dslash_roofline(S, ctx, vol, mixed, dims, ncols_total):
-    """The Wilson hopping kernel timed live on the library's stream: one launch
-    over all CG columns, and the shapes the CG graphs issue (one per concurrent
-    column branch; in FP64 those run in fixed-point integer arithmetic)."""
+def dslash_roofline(S, ctx, vol, mixed, dims, ncols_total, seed=None):
+    """The kernels of a CG iteration's operator, timed live on the library's stream: one
+    launch over all CG columns, and the shapes the CG graphs issue (one per concurrent
+    column branch).  FP64: D^H D in fixed-point integer arithmetic, against the rate of
+    the integer multiply-adds.  seed: (steps, ms) of the last seed phase."""
     shapes = cg_branch_cols(ncols_total)
     if not mixed:
-        k_ms = S.seed_time_operator(ctx, 1, ncols_total, 200)
-        flops = FLOPS_PER_SITE_D * vol * ncols_total
-        achieved = flops / (k_ms * 1e-3) / 1e12
-        peak = FP64_PEAK_GFLOPS / 1e3
-        probe = S.seed_time_fma(S.SEED_F64)["tflops"]
+        def fixed(cols):
+            ms = S.seed_time_operator(ctx, 0, cols, 200)
+            return ms, 2 * INT_MADS_PER_SITE_D * vol * cols / (ms * 1e-3) / 1e9
         shape_t = {}
         for c in sorted(set(shapes)):
-            m = S.seed_time_operator(ctx, 0, c, 200)
-            a = 2 * FLOPS_PER_SITE_D * vol * c / (m * 1e-3) / 1e12
-            shape_t[str(c)] = {"ms_per_apply": round(m, 5), "fp64_equivalent_tflops": round(a, 4)}
-        return {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak, 4), "unit": "TFLOP/s",
-                "frac": round(achieved / peak, 4),
-                "traffic": dslash_traffic() if tuple(dims) == WL["dims"] and ncols_total == 11 else None,
-                "kernel": "k_dslash<+1> (Wilson D in FP64 instructions, the form of a small lattice's seed steps), "
-                          "%d columns in one launch" % ncols_total,
-                "ms_per_launch": round(k_ms, 5), "flops_per_launch": flops,
-                "flops_per_site": FLOPS_PER_SITE_D,
+            m, a = fixed(c)
+            shape_t[str(c)] = {"ms_per_apply": round(m, 5), "achieved": round(a, 1), "frac": round(a / INT_MAD_PEAK_G, 4)}
+        k_ms, achieved = fixed(ncols_total)
+        # beside it: FP64 instructions, the form of a small lattice's seed steps and of its D and D^H by themselves
+        d_ms = S.seed_time_operator(ctx, 1, ncols_total, 200)
+        d_tf = FLOPS_PER_SITE_D * vol * ncols_total / (d_ms * 1e-3) / 1e12
+        peak = FP64_PEAK_GFLOPS / 1e3
+        probe = S.seed_time_fma(S.SEED_F64)["tflops"]
+        fp64 = {"kernel": "k_dslash<+1> (Wilson D in FP64 instructions), %d columns in one launch; no solve launches this "
+                          "shape" % ncols_total,
+                "ms_per_launch": round(d_ms, 5), "achieved": round(d_tf, 4), "peak": round(peak, 4), "unit": "TFLOP/s",
+                "frac": round(d_tf / peak, 4), "flops_per_site": FLOPS_PER_SITE_D,
                 "epilogue_flops_per_site": FLOPS_PER_SITE_D_EPILOGUE,
-                "frac_with_epilogue": round((FLOPS_PER_SITE_D + FLOPS_PER_SITE_D_EPILOGUE) * vol * ncols_total /
-                                            (k_ms * 1e-3) / 1e12 / peak, 4),
-                "launch_shapes": {"operator": "D^H D as the CG runs it (k_dslash_fix: integer arithmetic, conversion of "
-                                              "its input included)", "cg_branches": shapes, "per_shape": shape_t},
+                "traffic": dslash_traffic() if tuple(dims) == WL["dims"] and ncols_total == 11 else None,
                 "peak_note": "FP64 pipe from unit counts: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz",
                 "fp64_instructions_per_site": FP64_INSTR_PER_SITE_D,
                 "instruction_mix_ceiling": round(FLOPS_PER_SITE_D / (2.0 * FP64_INSTR_PER_SITE_D), 4),
-                "frac_of_instruction_mix_ceiling": round(achieved / peak / (FLOPS_PER_SITE_D /
-                                                                             (2.0 * FP64_INSTR_PER_SITE_D)), 4),
-                "peak_measured_probe": round(probe, 4), "frac_of_probe": round(achieved / probe, 4),
+                "peak_measured_probe": round(probe, 4),
                 "probe": "seed_time_fma(SEED_F64): FMA chains over the whole GPU, this run",
                 "fp64_matrix_probe": {k: round(v, 4) for k, v in S.seed_time_fp64_paths().items()}}
+        if seed and vol < 16384:   # the seed phase's own rate: its D and D^H over its whole time
+            a = seed[0] * 2 * FLOPS_PER_SITE_D * vol / (seed[1] * 1e-3) / 1e12
+            fp64["seed_phase"] = {"kernel": "k_seed_run_wilson (and the block flushes and reorthogonalizations)",
+                                  "steps": seed[0], "ms": round(seed[1], 3), "operator_tflops": round(a, 4),
+                                  "frac": round(a / peak, 4)}
+        return {"bound": "alu", "achieved": round(achieved, 1), "peak": round(INT_MAD_PEAK_G, 1), "unit": "GMAD/s",
+                "frac": round(achieved / INT_MAD_PEAK_G, 4), "traffic": None,
+                "kernel": "k_dslash_fix (Wilson D^H D in fixed-point arithmetic, the conversion of its input included), "
+                          "%d columns in one launch" % ncols_total,
+                "ms_per_apply": round(k_ms, 5), "mads_per_apply": 2 * INT_MADS_PER_SITE_D * vol * ncols_total,
+                "launch_shapes": {"cg_branches": shapes, "per_shape": shape_t},
+                "peak_note": "32 x 32 -> 64 bit multiply-adds at the measured 61 per clock and SM, 152 SMs, 2.07 GHz",
+                "fp64_instructions": fp64}
     k_ms = S.seed_time_operator(ctx, 4, ncols_total, 200)
     b = wilson_bytes(vol, ncols_total, fp32=True)
     achieved = b / (k_ms * 1e-3) / 1e9
@@ -755,7 +769,7 @@ def run_ours(args):
     ok = all(i["converged"] for i in i1[:1] + i2[1:])
     launches = st1["kernel_launches"] - st0["kernel_launches"]
 
-    roof = dslash_roofline(S, ctx, vol, mixed, dims, nrhs - 1)
+    roof = dslash_roofline(S, ctx, vol, mixed, dims, nrhs - 1, (i1[0]["iters"], st1["ms_seed"]))
 
     # end to end through the public API, host buffers (pinned), copies inside the timed region
     e2e = None
