@@ -566,8 +566,8 @@ void launch_dslash_fix(const WilsonFix &op, int sign, const int4 *in, const int3
     }
   } else if (dot != nullptr) {   // lockstep CG: q = D^H t
     FIX_GO(-1, 2);
-  } else if (sign > 0) {
-    FIX_GO(+1, 1);
+  } else if (sign > 0) {   // D by itself: from 16384 sites on only, never few
+    k_dslash_fix<+1, 1><<<grid, FT, kFixStage, s>>>(op, in, ein, ldq, qout, eout, out, ldo, items, ncols, col_active, d);
   } else {
     FIX_GO(-1, 1);
   }
