@@ -396,9 +396,14 @@ int32_t *fix_Te(seed_ctx *ctx) { return ctx->Fe + ctx->ldv / 12 * ctx->cap_cols;
 // seed system take this form: they amplify a last-bit change of A v_i until the late basis
 // vectors, and through the Galerkin projection the error (not the size) of the seeded
 // solutions, differ by a per cent.  Measured as the change of x^2.. (12 point sources, CG to 1e-8)
-// when b changes in its last bit: 3e-10 to 1e-9 on 6 x 8^3, 8^4 and 8^3 x 12, 4e-13 on 8^3
-// x 16, 5e-14 on 12^4 and below 1e-13 on 16^4; so from kFixSeedSites on they take the
-// fixed-point operator (apply_seed).
+// when b changes in its last bit, all in FP64 arithmetic, links exp(0.3 i H) with random Hermitian
+// H, kappa 0.155, reorthogonalization every 100 steps (250 to 280 steps): 2e-10 to 1e-9 on 6 x 8^3, 8^4
+// and 8^3 x 12, 2e-13 to 4e-13 on 8^3 x 16, 1e-14 on 8 x 12^3, 4e-14 on 12^4, 1e-15 on 8^2 x 16^2
+// and 16^4.  From kFixSeedSites on, with room above the largest of these that shows it, they
+// take the fixed-point operator (apply_seed).  The cause is the number of steps and how long the
+// basis goes without reorthogonalization, not the volume: at kappa 0.165 (185 steps) only 8^4 shows
+// it (1e-10), and near the critical kappa (0.14, 700 to 1000 steps) every lattice up to 16^4 does, by 3e-10
+// (every 25 steps) to 3e-5 (100): there solutions agree to CG's tolerance only, in either arithmetic.
 constexpr int64_t kFixSeedSites = 16384;
 bool fix_seed(const seed_ctx *ctx) { return ctx->kind == 1 && ctx->wfix.sites >= kFixSeedSites; }
 int apply_A64(seed_ctx *ctx, const void *X, int64_t ldx, void *Y, int64_t ldy, int ncols) {
@@ -1732,8 +1737,8 @@ struct StreamScope {
   }
 };
 
-// The operator by itself runs on the caller's stream, without the two event waits of StreamScope (D^H D
-// on 2048^2 CSR rows 60.6 -> 59.4 us a call).  Every other call starts
+// The operator by itself runs on the caller's stream, without the two event waits of StreamScope (a CSR
+// product on 2048^2 rows, one call after another: 65.5 -> 59.6 us).  Every other call starts
 // behind that stream; what frees work space without starting there waits for ev_apply.
 // Under a capture nothing is recorded for replays to come: work space that the graph
 // names is kept until seed_destroy (ensure_cols).

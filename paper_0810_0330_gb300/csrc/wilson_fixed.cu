@@ -8,13 +8,14 @@
 // L1.  Bound by instruction issue and the latency between dependent integer
 // instructions (0.39 instructions per clock and scheduler; long-scoreboard and fixed-latency
 // waits in equal parts; L2 at 20 %, DRAM at 1.5 TB/s).  D^H D with the
-// conversion of the input, GB300, FP64 kernel -> this one: 16^4 x 12 columns 2200 ->
-// 591 us, x 1 column 200 -> 71 us; 8^4 x 12 columns 160 -> 54 us.  Other splits
-// at 16^4 x 12: one thread per site 623 us (168 registers, waiting for memory two
-// thirds of the time); one per site and direction 808 us (an exchange of 24 KB of
-// partial sums per tile); 16 warps an SM instead of 12 (128 registers) 629 us; the links
-// fetched ahead as well (246 registers) 719 us; warps of a block kept in step
-// by a barrier per hop 612 us.
+// conversion of the input, GB300, FP64 kernel -> this one: 16^4 x 12 columns 2198 ->
+// 597 us, x 1 column 201 -> 72 us; 8^4 x 12 columns 160 -> 54 us; with the links' conversion
+// too (a seed_apply call) 16^4 x 12 columns 2198 -> 620 us.  Other splits, such calls at 16^4 x 12
+// columns, beside 613 us of this one in that session: one thread per site 623 us (168
+// registers, waiting for memory two thirds of the time); one per site and direction 808 us (an
+// exchange of 24 KB of partial sums per tile); 16 warps an SM instead of 12 (128 registers) 629 us;
+// the links fetched ahead as well (246 registers) 719 us; warps of a block kept in step
+// by a barrier per hop 612 us (no gain).
 #include "seed_device.cuh"
 #include "wilson_fixed.cuh"
 
