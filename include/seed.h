@@ -120,7 +120,7 @@ typedef struct {
                              0 (default): the seed's runs of Lanczos steps between
                              reorthogonalizations in one persistent cooperative kernel (when the
                              frequency is 0 or >= 8; not in FP64 on Wilson lattices from 16384
-                             sites on), everything else as step kernels
+                             sites on while there is memory for the fixed-point operator), everything else as step kernels
                              replayed from CUDA graphs, the lockstep CG in up to three concurrent
                              column branches; small real CSR problems in FP64 (n <= 9728) run
                              the whole seed run as one cooperative kernel when the frequency is
